@@ -363,7 +363,147 @@ __device__ __forceinline__ void hop_dir_raw(f2 (&acc)[12], const f2 (&ps)[12], c
   }
 }
 
-// FP64 version of hop_dir with the sign S at run time
+// ------------------------------------------------------------------ FP64 hop in fixed point
+//
+// GB300 issues two FP64 operations per clock and SM but sixty 32 x 32 + 64 bit integer
+// multiply-adds (measured: DFMA 1.99, DADD 1.67, IMAD.WIDE 60 per clock and SM), so the
+// FP64 hop forms its SU(3) products in integers.  Per (site, s) the projected half-spinors h
+// are formed in FP64 as before (Eq. 12), then brought to the exponent E = the largest among
+// the neighbours so far (plus one bit, so that E seldom has to grow): h = V 2^(E - 1080),
+// |V| < 2^58.  Links are in units of 2^-60.  Both are split into 30-bit halves that carry the
+// sign, V = hi 2^30 + lo, and a product sum over the six real terms of a row is
+//   sum W V / 2^60 = sum Wh Vh + (sum (Wh Vl + Wl Vh)) / 2^30,
+// three 64-bit multiply-adds per real product; the dropped Wl Vl are below one unit each.
+// Bounds: a link row's 2-norm is at most sqrt(1.01) (checked; SU(3) rows have norm 1), so a
+// row's result is below sqrt(1.01 * 6) 2^58 < 2^59.4 and the sum over eight directions below
+// 2^62.4; the cross terms are below 6 (2^60 + 2^58) < 2^63.  An error of about one unit per
+// direction is 2^-56 of the largest |h|: below FP64's own rounding of the same sums
+// (2^-53 of each partial sum).  Links or neighbours outside the bounds (not finite, or
+// exponents outside [FX_EMIN, FX_EMAX]) take the FP64 arithmetic (hop_site_f64).
+// Neighbour sums therefore do not depend on the order of the sites of a tile or on whether a
+// neighbour is stored as a spinor or, in a halo slot, as its projection.
+
+constexpr int FX_EMIN = 80, FX_EMAX = 2000;
+// int4 per site of the fixed-point links: 8 links x 9 entries {re hi, re lo, im hi, im lo}, and
+// one of padding, so that the sites of a warp read from different banks
+constexpr int FX_SITE_I4 = 73;
+
+// V = x 2^(1075 + L - E), truncated, as V = hi 2^30 + lo; E is at least x's exponent field (an x
+// above it gives 0, and so do FP64 zeros and denormals)
+template <int L>
+__device__ __forceinline__ void to_fixed(double x, int E, int &hi, int &lo) {
+  const int xh = __double2hiint(x);
+  const unsigned mh = (xh & 0xfffff) | 0x100000;
+  const unsigned sh = min((unsigned)(E - ((xh >> 20) & 0x7ff)), 63u);
+  const unsigned long long m = ((unsigned long long)mh << 32 | (unsigned)__double2loint(x)) << L >> sh;
+  const int sg = (xh >> 31) | 1;
+  hi = (int)(m >> 30) * sg;
+  lo = (int)(m & 0x3fffffffu) * sg;
+}
+
+__device__ __forceinline__ long long mul_w(int a, int b) { return (long long)a * b; }
+__device__ __forceinline__ void mad_w(long long &c, int a, int b) {
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(c) : "r"(a), "r"(b));
+}
+
+// h_j = psi_up + S A psi_dn of direction MU (spin projection), FP64
+template <int MU, int S>
+__device__ __forceinline__ void project_f64(const double (&ps)[24], double (&h)[12]) {
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const int src = 2 * (a + 3 * (2 + a_col(MU, j))), dst = 2 * (a + 3 * j);
+      // phase code 0: 1, 1: i, 2: -1, 3: -i
+      const int p = a_ph(MU, j);
+      const double vr = (p & 1) ? ps[src + 1] : ps[src], vi = (p & 1) ? ps[src] : ps[src + 1];
+      h[dst] = (p == 1 || p == 2) == (S > 0) ? ps[dst] - vr : ps[dst] + vr;
+      h[dst + 1] = (p == 2 || p == 3) == (S > 0) ? ps[dst + 1] - vi : ps[dst + 1] + vi;
+    }
+}
+
+// acc += (1 + S g_MU) W psi in units of 2^(E - 1080); W: the link's nine entries; returns
+// false if a value is outside the fixed-point range (acc is then meaningless)
+template <int MU, int S>
+__device__ __forceinline__ bool hop_dir_fixed(long long (&acc)[24], int &E, const double (&ps)[24], const int4 *W) {
+  double h[12];
+  project_f64<MU, S>(ps, h);
+  int em = 0;
+#pragma unroll
+  for (int q = 0; q < 12; ++q) em = max(em, __double2hiint(h[q]) & 0x7fffffff);
+  em >>= 20;
+  bool ok = em <= FX_EMAX;
+  if (em < FX_EMIN) {  // all zero (nothing to add), or too small for the fixed-point range
+    unsigned any = 0;
+#pragma unroll
+    for (int q = 0; q < 12; ++q) any |= (unsigned)(__double2hiint(h[q]) << 1) | (unsigned)__double2loint(h[q]);
+    ok = any == 0;
+  }
+  if (em > E) {
+    const int d = min(em + 1 - E, 63);
+#pragma unroll
+    for (int c = 0; c < 24; ++c) acc[c] >>= d;
+    E = em + 1;
+  }
+  int ph[6], pl[6], qh[6], ql[6], nh[6], nl[6];  // real parts, imaginary parts, - imaginary parts
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    to_fixed<5>(h[2 * q], E, ph[q], pl[q]);
+    to_fixed<5>(h[2 * q + 1], E, qh[q], ql[q]);
+    nh[q] = -qh[q];
+    nl[q] = -ql[q];
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int4 w0 = W[3 * a], w1 = W[3 * a + 1], w2 = W[3 * a + 2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      long long Hr = 0, Hi = 0, Xr = 1 << 29, Xi = 1 << 29;
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const int4 w = b == 0 ? w0 : b == 1 ? w1 : w2;
+        const int q = 3 * j + b;
+        mad_w(Hr, w.x, ph[q]), mad_w(Hr, w.z, nh[q]);
+        mad_w(Hi, w.x, qh[q]), mad_w(Hi, w.z, ph[q]);
+        mad_w(Xr, w.x, pl[q]), mad_w(Xr, w.y, ph[q]), mad_w(Xr, w.z, nl[q]), mad_w(Xr, w.w, nh[q]);
+        mad_w(Xi, w.x, ql[q]), mad_w(Xi, w.y, qh[q]), mad_w(Xi, w.z, pl[q]), mad_w(Xi, w.w, ph[q]);
+      }
+      const long long re = Hr + (Xr >> 30), im = Hi + (Xi >> 30);
+      const int u = 2 * (a + 3 * j);
+      acc[u] += re;
+      acc[u + 1] += im;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        if (ad_col(MU, k) != j) continue;
+        const int dn = 2 * (a + 3 * (2 + k)), p = ad_ph(MU, k);
+        // S phase (re + i im): phase 0: 1, 1: i, 2: -1, 3: -i
+        const bool neg_r = (p == 1 || p == 2) == (S > 0), neg_i = (p == 2 || p == 3) == (S > 0);
+        const long long vr = (p & 1) ? im : re, vi = (p & 1) ? re : im;
+        acc[dn] = neg_r ? acc[dn] - vr : acc[dn] + vr;
+        acc[dn + 1] = neg_i ? acc[dn + 1] - vi : acc[dn + 1] + vi;
+      }
+    }
+  }
+  return ok;
+}
+
+// a link row (three complex entries) in units of 2^-60, split as above; false if its 2-norm is
+// out of bounds or not a number
+__device__ __forceinline__ bool link_row_fixed(const double *w, int4 *o) {
+  float n2 = 0.f;
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    const double re = w[2 * b], im = w[2 * b + 1];
+    n2 += (float)re * (float)re + (float)im * (float)im;
+    int4 v;
+    to_fixed<8>(re, 1023, v.x, v.y);
+    to_fixed<8>(im, 1023, v.z, v.w);
+    o[b] = v;
+  }
+  return n2 <= 1.01f;
+}
+
+// the same in plain FP64 with the sign S at run time, for values out of the fixed-point range
 template <int MU, typename R>
 __device__ __forceinline__ void hop_dir_s(R (&acc)[24], const R (&ps)[24], const R (&W)[18], R S) {
   R h[2][3][2];

@@ -232,17 +232,13 @@ bool build_matrices(dwf_ctx *c) {
   return true;
 }
 
-// M5 and M5^T of Eq. 8 as recurrences along s, for the hop epilogues.  With
-// A = (d - m0) sqrt(omega) (1 + cL) + omega^{-1/2} (1 - L) (cyclic bidiagonal through the
-// corner kappa of L, Eq. 4) and P = sqrt(omega) (1 + cL): M5 = P A^{-1}, M5^T = A^{-T} P^T.
-// A chirality's recurrence visits s in one direction (step j at s = j, or Ns - 1 - j when
-// backward: chirality - for M5, chirality + for M5^T); every step uses the values of the
-// step before it, and step 0 those of the last step scaled by kappa:
-//   g_j = PS_j v_j + PN_j vp,  z_j = (g_j - BB_j zp) AI_j,  u_j = QS_j z_j + QN_j zp,
-// with the first zp = kappa z_last from the closure z_last = sum_j W_j v_j and the first
-// vp = kappa v_last.  Table: per chirality, RC_N reals per step.
-enum { RC_PS, RC_PN, RC_BB, RC_AI, RC_QS, RC_QN, RC_W, RC_N = 8 };
-
+// The fifth-dimension matrices as recurrences along s for the FP64 kernels (tables of RC_A).
+// With A = (d - m0) sqrt(omega) (1 + cL) + omega^{-1/2} (1 - L) (cyclic bidiagonal through the
+// corner kappa of L, Eq. 4; diagonal a, below it beta) and P = sqrt(omega) (1 + cL):
+// M5 = P A^{-1}, M5^T = A^{-T} P^T (Eq. 8), S1 = M5 omega^{-1/2}, S2 = (1 + cL)^{-1}
+// omega^{-1/2} (Eq. 9).  A chirality's recurrence visits s in one direction (step j at s = j, or
+// Ns - 1 - j when backward: chirality - , or chirality + for M5^T).  In P A^{-1} the solved z
+// is kept as sqrt(omega) z, which leaves one multiplication per step for P.
 void apply_recurrence(const double *T, int Ns, bool bwd, double kappa, const double *v, double *u) {
   auto sg = [&](int j) { return bwd ? Ns - 1 - j : j; };
   double zc = 0.0;
@@ -251,15 +247,15 @@ void apply_recurrence(const double *T, int Ns, bool bwd, double kappa, const dou
   for (int j = 0; j < Ns; ++j) {
     const double *t = T + j * RC_N;
     const int s = sg(j);
-    const double g = t[RC_PS] * v[s] + t[RC_PN] * vp;
-    const double z = (g - t[RC_BB] * zp) * t[RC_AI];
-    u[s] = t[RC_QS] * z + t[RC_QN] * zp;
+    const double z = t[RC_A] * v[s] + t[RC_B] * vp - t[RC_C] * zp;
+    u[s] = z + t[RC_R] * zp;
     zp = z;
     vp = v[s];
   }
 }
 
-// builds the tables and checks each against the dense M5 / M5^T column by column
+// builds the tables and checks each against its dense matrix column by column; M5 and M5^T
+// have to agree, the others are left to the dense kernel where they do not
 bool build_recurrences(dwf_ctx *c) {
   const int Ns = c->Ns;
   const double kappa = -c->mq / (2.0 * c->m0);
@@ -270,60 +266,64 @@ bool build_recurrences(dwf_ctx *c) {
     a[s] = dm * sw[s] + 1.0 / sw[s];
     beta[s] = dm * c->sigma[s] / sw[s] - 1.0 / sw[s];
     cc[s] = c->sigma[s] / c->omega[s];
+    if (a[s] == 0.0) return false;
   }
-  for (int tr = 0; tr < 2; ++tr) {
-    c->rec[tr].assign((size_t)2 * Ns * RC_N, 0.0);
-    for (int chi = 0; chi < 2; ++chi) {
-      const bool bwd = (chi ^ tr) != 0;
+  const int kinds[] = {MK_M5, MK_M5T, MK_S1, MK_S2};
+  for (int kind : kinds) {
+    std::vector<double> &rec = c->rec[kind];
+    rec.assign((size_t)2 * Ns * RC_N, 0.0);
+    bool ok = true;
+    for (int chi = 0; chi < 2 && ok; ++chi) {
+      const bool bwd = (chi ^ (kind == MK_M5T)) != 0;
       auto sg = [&](int j) { return bwd ? Ns - 1 - j : j; };
-      double *T = c->rec[tr].data() + (size_t)chi * Ns * RC_N;
+      double *T = rec.data() + (size_t)chi * Ns * RC_N;
       for (int j = 0; j < Ns; ++j) {
         const int s = sg(j), n = sg((j + Ns - 1) % Ns);  // this step's s and the step before's
         double *t = T + j * RC_N;
-        if (a[s] == 0.0) return false;
-        t[RC_AI] = 1.0 / a[s];
-        if (tr == 0) {  // M5 = P A^{-1}: solve, then u = sqrt(omega) (z + c L z)
-          t[RC_PS] = 1.0;
-          t[RC_PN] = 0.0;
-          t[RC_BB] = beta[s];
-          t[RC_QS] = sw[s];
-          t[RC_QN] = sw[s] * cc[s];
-        } else {  // M5^T = A^{-T} P^T: g = P^T v, then solve with A^T
-          t[RC_PS] = sw[s];
-          t[RC_PN] = sw[n] * cc[n];
-          t[RC_BB] = beta[n];
-          t[RC_QS] = 1.0;
-          t[RC_QN] = 0.0;
+        if (kind == MK_M5T) {  // g = P^T v, then A^T z = g
+          t[RC_A] = sw[s] / a[s];
+          t[RC_B] = sw[n] * cc[n] / a[s];
+          t[RC_C] = beta[n] / a[s];
+        } else if (kind == MK_S2) {  // (1 + cL) z = omega^{-1/2} v
+          t[RC_A] = 1.0 / sw[s];
+          t[RC_C] = cc[s];
+        } else {  // A z = v (S1: omega^{-1/2} v), u = sqrt(omega) (z + c L z); sqrt(omega) z kept
+          t[RC_A] = (kind == MK_S1 ? 1.0 : sw[s]) / a[s];
+          t[RC_C] = beta[s] / a[s] * sw[s] / sw[n];
+          t[RC_R] = cc[s] * sw[s] / sw[n];
         }
       }
-      // closure: z_last = sum_j lam_j g_j (forward substitution with z depending linearly on
-      // z_last through step 0), and g_j = PS_j v_j + PN_j vp_j gives the weights on v
-      double q = -T[RC_BB] * kappa * T[RC_AI];
-      for (int j = 1; j < Ns; ++j) q = -T[j * RC_N + RC_BB] * q * T[j * RC_N + RC_AI];
+      // closure: z_last depends linearly on z_{-1} = kappa z_last through every step
+      double q = -T[RC_C] * kappa;
+      for (int j = 1; j < Ns; ++j) q *= -T[j * RC_N + RC_C];
       const double den = 1.0 - q;
-      if (den == 0.0) return false;
+      ok = den != 0.0;
       double r = 1.0;
-      for (int j = Ns - 1; j >= 0; --j) {
-        lam[j] = T[j * RC_N + RC_AI] * r / den;
-        r *= -T[j * RC_N + RC_BB] * T[j * RC_N + RC_AI];
+      for (int j = Ns - 1; j >= 0 && ok; --j) {
+        lam[j] = r / den;
+        r *= -T[j * RC_N + RC_C];
       }
-      for (int j = 0; j < Ns; ++j) {
-        double w = lam[j] * T[j * RC_N + RC_PS];
-        if (j + 1 < Ns) w += lam[j + 1] * T[(j + 1) * RC_N + RC_PN];
-        if (j == Ns - 1) w += kappa * lam[0] * T[RC_PN];
+      for (int j = 0; j < Ns && ok; ++j) {
+        double w = lam[j] * T[j * RC_N + RC_A];
+        if (j + 1 < Ns) w += lam[j + 1] * T[(j + 1) * RC_N + RC_B];
+        if (j == Ns - 1) w += kappa * lam[0] * T[RC_B];
         T[j * RC_N + RC_W] = w;
       }
       // check: the recurrence reproduces every column of the dense matrix
-      const double *M = c->mat[tr ? MK_M5T : MK_M5].data() + (size_t)chi * Ns * Ns;
+      const double *M = c->mat[kind].data() + (size_t)chi * Ns * Ns;
       double mmax = 0.0;
       for (int i = 0; i < Ns * Ns; ++i) mmax = std::max(mmax, fabs(M[i]));
-      for (int t0 = 0; t0 < Ns; ++t0) {
+      for (int t0 = 0; t0 < Ns && ok; ++t0) {
         std::fill(v.begin(), v.end(), 0.0);
         v[t0] = 1.0;
         apply_recurrence(T, Ns, bwd, kappa, v.data(), u.data());
         for (int s = 0; s < Ns; ++s)
-          if (!(fabs(u[s] - M[s * Ns + t0]) <= 1e-11 * mmax)) return false;
+          if (!(fabs(u[s] - M[s * Ns + t0]) <= 1e-11 * mmax)) ok = false;
       }
+    }
+    if (!ok) {
+      if (kind == MK_M5 || kind == MK_M5T) return false;
+      rec.clear();
     }
   }
   return true;
@@ -560,7 +560,7 @@ const void *dmat(dwf_ctx *c, int prec, int kind) { return c->dmat[mat_index(prec
 // recurrence table (FP64)
 void set_m5(HopArgs &a, dwf_ctx *c, int prec, bool trans) {
   a.K = dmat(c, prec, trans ? MK_M5T : MK_M5);
-  a.rec = c->drec[mat_index(prec)][trans ? 1 : 0];
+  a.rec = c->drec[trans ? MK_M5T : MK_M5];
   a.mtrans = trans ? 1 : 0;
   a.kappa = -c->mq / (2.0 * c->m0);
 }
@@ -827,18 +827,13 @@ dwf_status dwf_create(const int dims[4], int Ns, double m0, double mq, const dou
       return bail(e);
     if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return bail(e);  // kd, kf are reused
   }
-  for (int tr = 0; tr < 2; ++tr) {
-    const size_t nr = c->rec[tr].size();
-    std::vector<float> rf(c->rec[tr].begin(), c->rec[tr].end());
-    if ((e = dmalloc(&c->drec[0][tr], nr * sizeof(double), c->device, c->stream)) != cudaSuccess) return bail(e);
-    if ((e = dmalloc(&c->drec[1][tr], nr * sizeof(float), c->device, c->stream)) != cudaSuccess) return bail(e);
-    if ((e = cudaMemcpyAsync(c->drec[0][tr], c->rec[tr].data(), nr * sizeof(double), cudaMemcpyHostToDevice,
-                             c->stream)) != cudaSuccess)
-      return bail(e);
-    if ((e = cudaMemcpyAsync(c->drec[1][tr], rf.data(), nr * sizeof(float), cudaMemcpyHostToDevice, c->stream)) !=
+  for (int k = 0; k < MK_COUNT; ++k) {
+    const size_t nr = c->rec[k].size();
+    if (!nr) continue;
+    if ((e = dmalloc((void **)&c->drec[k], nr * sizeof(double), c->device, c->stream)) != cudaSuccess) return bail(e);
+    if ((e = cudaMemcpyAsync(c->drec[k], c->rec[k].data(), nr * sizeof(double), cudaMemcpyHostToDevice, c->stream)) !=
         cudaSuccess)
       return bail(e);
-    if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return bail(e);  // rf is a temporary
   }
   Geom g = geom(c);
   for (int p = 0; p < 2; ++p) {
@@ -876,8 +871,7 @@ dwf_status dwf_destroy(dwf_ctx *c) {
     }
     for (auto &row : c->dmat)
       for (void *p : row) dfree(p, c->stream);
-    for (auto &row : c->drec)
-      for (void *p : row) dfree(p, c->stream);
+    for (double *p : c->drec) dfree(p, c->stream);
     release_gauge(c);
     dfree(c->d_Ug, c->stream);
     for (int *p : c->d_nbr) dfree(p, c->stream);

@@ -69,9 +69,9 @@ struct dwf_ctx {
   std::vector<double> mat[dwf::MK_COUNT];
   // device matrices per arithmetic precision (0: double, 1: float), kernel order
   void *dmat[2][dwf::MK_COUNT] = {};
-  // M5 (0) and M5^T (1) as recurrence tables along s (host FP64; device per precision)
-  std::vector<double> rec[2];
-  void *drec[2][2] = {};
+  // M5, M5^T, S1 and S2 as FP64 recurrence tables along s (RC_A); empty where there is none
+  std::vector<double> rec[dwf::MK_COUNT];
+  double *drec[dwf::MK_COUNT] = {};
   int *d_nbr[2] = {nullptr, nullptr};
   double *d_U = nullptr;  // FP64 host-layout copy of the gauge field
   void *d_gauge[4][2] = {};

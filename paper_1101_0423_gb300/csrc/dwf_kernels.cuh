@@ -191,13 +191,23 @@ template <int EPI> struct EpiT {
   static constexpr bool has_red = EPI == E_XPAY_G5 || EPI == E_CG_UPDATE || EPI == E_RESID;
 };
 
+// FP64 recurrence along s (one table per matrix: per chirality Ns steps, step j at s = j, or
+// Ns - 1 - j for a chirality that runs backward), two or three FP64 operations a real and step
+// and one for the closure, against Ns for the dense row:
+//   z_j = A_j v_j + B_j v_{j-1} - C_j z_{j-1},  u_j = z_j + R_j z_{j-1},
+// where step 0 takes v_{-1} = kappa v_{Ns-1} and z_{-1} = kappa z_{Ns-1}, with z_{Ns-1} known
+// beforehand from the closure z_{Ns-1} = sum_j W_j v_j
+enum { RC_A, RC_B, RC_C, RC_R, RC_W, RC_N = 6 };
+// which coefficients a table has: B = 0 (M5, S1, S2) or R = 0 (M5^T)
+enum { REC_SOLVE_MUL = 0, REC_MUL_SOLVE = 1 };
+
 struct HopArgs {
   Field in, out, y, b, r;
   const void *gauge;   // doubled gauge of the output parity: [cb][SITE_LREALS], links [8][LREALS]
   const int *nbr;      // [cb][8] for the output parity
   const void *K;       // FP32 arithmetic: M5 or M5^T, dense, kernel order K[chi][t][s]
   const void *rec;     // FP64: the same as a recurrence table along s, per chirality Ns
-                       // steps of {PS, PN, BB, AI, QS, QN, W, 0}
+                       // steps of RC_N reals (see RC_A)
   int mtrans;          // 0: M5, 1: M5^T (direction of each chirality's recurrence)
   double kappa;        // corner of L, -mq / (2 m0) (Eq. 4)
   double coef;         // scale of H (plain/xpay) or of the matrix (M5 epilogues)
@@ -235,12 +245,12 @@ __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes) {
 __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~size_t(15); }
 
 // dynamic shared memory of k_hop, in bytes:
-//   [mbarriers, 64][links as copied] x nb [neighbour indices] x nb [16-bit links expanded][M]
+//   [mbarriers, 64][links as copied] x nb [neighbour indices] x nb [links expanded][M]
 // with nb = 2 when a persistent CTA receives the next tile while computing this one, else 1
-// (links and indices arrive by TMA bulk copies).  FP32 and FP64 kernels use the links as
-// copied (FP32 links are padded to 80 bytes, so the nine complex entries are five aligned
-// float4); the 16-bit forms rebuild each link's third row and expand the tile's links into
-// that same FP32 form.  The M5 staging rows overlay everything from offset 64 on (kernels
+// (links and indices arrive by TMA bulk copies).  FP32 kernels use the links as copied (padded
+// to 80 bytes, so the nine complex entries are five aligned float4); the 16-bit forms rebuild
+// each link's third row and expand the tile's links into that same FP32 form; FP64 kernels
+// convert them to fixed point once for the Ns threads of a site.  The M5 staging rows overlay everything from offset 64 on (kernels
 // with an M5 epilogue take one tile per CTA, so the link buffers are dead by then).  Shared
 // memory is kept small on purpose: what the CTAs leave of the SM's 256 KB is the L1 that
 // holds the neighbour gathers in flight.
@@ -261,15 +271,17 @@ template <int P> struct HopSmem {
   // stores fall in distinct bank groups; sites padded by another 16 bytes
   static constexpr int ROW = 24 + 16 / (int)sizeof(RL);
   __host__ __device__ static size_t stage(int spb, int Ns) { return (size_t)spb * (Ns * ROW * sizeof(RL) + 16); }
-  // FP32 links are used as copied; the 16-bit forms are expanded
-  static constexpr bool EXPAND = F2 && P != P_F32;
+  // FP32 links are used as copied; the other forms are expanded
+  // (16-bit: to the FP32 form; FP64: to the fixed-point form)
+  static constexpr bool EXPAND = P != P_F32;
+  static constexpr int EXP_SITE_BYTES = 16 * (F2 ? LINK_SITE_F4 : FX_SITE_I4);
   __host__ __device__ static size_t off_k(int spb, int Ns, int nb, bool has_m) {
-    const size_t e = off_exp(spb, nb) + (EXPAND ? (size_t)spb * LINK_SITE_F4 * 16 : 0);
+    const size_t e = off_exp(spb, nb) + (EXPAND ? (size_t)spb * EXP_SITE_BYTES : 0);
     const size_t st = has_m ? 64 + stage(spb, Ns) : 0;
     return align16(e > st ? e : st);
   }
   // M5 / M5^T: dense (FP32 arithmetic) or a recurrence table of 2 chiralities x Ns steps x
-  // 8 reals (FP64).  Dense, even Ns: per chirality and t a row of Ns/2 pairs
+  // RC_N reals (FP64).  Dense, even Ns: per chirality and t a row of Ns/2 pairs
   // (K[b][t], K[b + Ns/2][t]), the second chirality kq_stride pairs after the first; odd Ns:
   // (k, k) pairs K[chi][t][s].
   __host__ __device__ static int kq_stride(int Ns) {
@@ -279,7 +291,7 @@ template <int P> struct HopSmem {
     return Ns * (Ns / 2) + ((16 - (Ns * Ns) % 32 + 32) % 32) / 2;
   }
   __host__ __device__ static size_t kbytes(int Ns) {
-    if (!F2) return (size_t)2 * Ns * 8 * sizeof(RL);
+    if (!F2) return (size_t)2 * Ns * RC_N * sizeof(RL);
     const size_t dense = (size_t)2 * Ns * Ns * 8, paired = (size_t)2 * kq_stride(Ns) * 8;
     return dense > paired ? dense : paired;
   }
@@ -317,12 +329,78 @@ __host__ __device__ inline size_t hop_smem_bytes(int spb, int Ns) {
   return HopSmem<P>::bytes(spb, Ns, hop_persistent<EPI>() ? 2 : 1, EpiT<EPI>::has_m);
 }
 
+// the recurrence of RC_A along one column of two reals, in place: col[0], col[step], ... are
+// its Ns values in the order of the steps
+__device__ __forceinline__ void s_recurrence(double2 *col, int step, const double *T, int Ns, double kappa, int form) {
+  double2 zp = make_double2(0.0, 0.0), vp = zp;
+#pragma unroll 4
+  for (int j = 0; j < Ns; ++j) {
+    vp = col[j * step];
+    const double w = T[j * RC_N + RC_W];
+    zp.x = fma(w, vp.x, zp.x);
+    zp.y = fma(w, vp.y, zp.y);
+  }
+  zp.x *= kappa, zp.y *= kappa;
+  if (form == REC_SOLVE_MUL) {
+#pragma unroll 4
+    for (int j = 0; j < Ns; ++j) {
+      const double2 ab = *reinterpret_cast<const double2 *>(T + j * RC_N), cr = *reinterpret_cast<const double2 *>(T + j * RC_N + 2);
+      const double2 v = col[j * step];
+      double2 z, u;
+      z.x = fma(-cr.x, zp.x, ab.x * v.x);
+      z.y = fma(-cr.x, zp.y, ab.x * v.y);
+      u.x = fma(cr.y, zp.x, z.x);
+      u.y = fma(cr.y, zp.y, z.y);
+      zp = z;
+      col[j * step] = u;
+    }
+  } else {
+    vp.x *= kappa, vp.y *= kappa;
+#pragma unroll 4
+    for (int j = 0; j < Ns; ++j) {
+      const double2 ab = *reinterpret_cast<const double2 *>(T + j * RC_N), cr = *reinterpret_cast<const double2 *>(T + j * RC_N + 2);
+      const double2 v = col[j * step];
+      zp.x = fma(-cr.x, zp.x, fma(ab.y, vp.x, ab.x * v.x));
+      zp.y = fma(-cr.x, zp.y, fma(ab.y, vp.y, ab.x * v.y));
+      vp = v;
+      col[j * step] = zp;
+    }
+  }
+}
+
+// the hop sum of one (site, s) in plain FP64 (fields or links out of the fixed-point range)
+template <int P>
+__device__ __noinline__ void hop_site_f64(const Field in, const int *nb, int s, int Ns, const double *links, double *out) {
+  double acc[24];
+#pragma unroll
+  for (int c = 0; c < 24; ++c) acc[c] = 0;
+  double ps[24], W[18];
+#pragma unroll
+  for (int d = 0; d < 8; ++d) {
+    load_sp_ro<P>(in, nb[d], s, Ns, ps);
+    load_link<P>(links + d * PT<P>::LREALS, W);
+    const double S = d < 4 ? -1.0 : 1.0;
+    switch (d & 3) {
+      case 0: hop_dir_s<0>(acc, ps, W, S); break;
+      case 1: hop_dir_s<1>(acc, ps, W, S); break;
+      case 2: hop_dir_s<2>(acc, ps, W, S); break;
+      default: hop_dir_s<3>(acc, ps, W, S); break;
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < 24; ++c) out[c] = acc[c];
+}
+
 // k_hop: one thread per (site, s), CTA = (Ns, spb) = one tile of spb sites (kernels without
 // an M5 epilogue: a grid of as many CTAs as fit on the GPU at once, walking all tiles).  Per
-// tile: eight gathers of the neighbours' spinors (Eq. 12), the hop sum in packed FP32 pairs
-// (or FP64), the epilogue.
+// tile: eight gathers of the neighbours' spinors (Eq. 12), the hop sum in packed FP32 pairs or
+// FP64 fixed point, the epilogue.  The FP64
+// forms (fixed-point products, FP64 projections and M5) are capped at 128 registers, four CTAs
+// per SM: a CTA's M5 phase keeps the FP64 pipe busy while others are in their integer hop
+// phase (C C^dag in FP64 at 16^3x32x16: 3.83 ms, against 4.05 ms with three CTAs of 168
+// registers, and 11.0 ms with the products in FP64).
 template <int P, int EPI, int NSC>
-__global__ void __launch_bounds__(256) k_hop(const HopArgs a) {
+__global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 1) k_hop(const HopArgs a) {
   // one right-hand side of a batch per grid row; fields are offset where they are used, so
   // the pointers stay in parameter space instead of registers
   const int rb = blockIdx.y;
@@ -409,12 +487,12 @@ __global__ void __launch_bounds__(256) k_hop(const HopArgs a) {
         }
       }
     } else {
-      // the matrix acts on coef H: coef scales g and the closure (entries PS, PN, W)
+      // the matrix acts on coef H: coef scales the entries that multiply v
       const R *Tg = static_cast<const R *>(a.rec);
       R *sT = reinterpret_cast<R *>(sKb);
-      for (int i = tid; i < 2 * Ns * 8; i += nthr) {
-        const int e = i & 7;
-        sT[i] = (e == 0 || e == 1 || e == 6) ? (R)(a.coef * (double)Tg[i]) : Tg[i];
+      for (int i = tid; i < 2 * Ns * RC_N; i += nthr) {
+        const int e = i % RC_N;
+        sT[i] = (e == RC_A || e == RC_B || e == RC_W) ? a.coef * Tg[i] : Tg[i];
       }
     }
   }
@@ -463,7 +541,16 @@ __global__ void __launch_bounds__(256) k_hop(const HopArgs a) {
         if (it > 0) prefetch_ops(tile);
       }
     }
-    if constexpr (SM::EXPAND) {
+    bool slow_tile = false;  // FP64: a link is out of the fixed-point range
+    if constexpr (!F2) {
+      bool bad = false;
+      int4 *sI = reinterpret_cast<int4 *>(sP);
+      for (int r = tid; r < nsite * 24; r += nthr) {
+        const int l = r / 24, row = r - 24 * l;
+        bad |= !link_row_fixed(sL + (size_t)l * T::SITE_LREALS + row * 6, sI + (size_t)l * FX_SITE_I4 + row * 3);
+      }
+      slow_tile = __syncthreads_or(bad);
+    } else if constexpr (SM::EXPAND) {
       // 16-bit links: rebuild row 3 and expand each link into the padded FP32 form
       for (int l = tid; l < nsite * 8; l += nthr) {
         float W[18];
@@ -511,21 +598,37 @@ __global__ void __launch_bounds__(256) k_hop(const HopArgs a) {
 #pragma unroll
         for (int q = 0; q < 12; ++q) upk2(ac2[q], acc[2 * q], acc[2 * q + 1]);
       } else {
+        long long ai[24];
 #pragma unroll
-        for (int c = 0; c < 24; ++c) acc[c] = 0;
-        const typename T::lreal *myL = sL + (size_t)sl * T::SITE_LREALS;
-        R ps[24], W[18];
+        for (int c = 0; c < 24; ++c) ai[c] = 0;
+        int ex = FX_EMIN;
+        bool ok = !slow_tile;
+        const int4 *myW = reinterpret_cast<const int4 *>(sP) + (size_t)sl * FX_SITE_I4;
 #pragma unroll
         for (int d = 0; d < 8; ++d) {
+          R ps[24];
           load_sp_ro<P>(F(a.in), nb[d], s, Ns, ps);
-          load_link<P>(myL + d * T::LREALS, W);
-          const R S = d < 4 ? (R)-1 : (R)1;
-          switch (d & 3) {
-            case 0: hop_dir_s<0>(acc, ps, W, S); break;
-            case 1: hop_dir_s<1>(acc, ps, W, S); break;
-            case 2: hop_dir_s<2>(acc, ps, W, S); break;
-            default: hop_dir_s<3>(acc, ps, W, S); break;
+          const int4 *W = myW + 9 * d;
+          switch (d) {
+            case 0: ok &= hop_dir_fixed<0, -1>(ai, ex, ps, W); break;
+            case 1: ok &= hop_dir_fixed<1, -1>(ai, ex, ps, W); break;
+            case 2: ok &= hop_dir_fixed<2, -1>(ai, ex, ps, W); break;
+            case 3: ok &= hop_dir_fixed<3, -1>(ai, ex, ps, W); break;
+            case 4: ok &= hop_dir_fixed<0, 1>(ai, ex, ps, W); break;
+            case 5: ok &= hop_dir_fixed<1, 1>(ai, ex, ps, W); break;
+            case 6: ok &= hop_dir_fixed<2, 1>(ai, ex, ps, W); break;
+            default: ok &= hop_dir_fixed<3, 1>(ai, ex, ps, W); break;
           }
+        }
+        if (ok) {
+          const R scale = __hiloint2double((ex - 57) << 20, 0);  // 2^(ex - 1080)
+#pragma unroll
+          for (int c = 0; c < 24; ++c) acc[c] = (R)ai[c] * scale;
+        } else {
+          R slow[24];
+          hop_site_f64<P>(F(a.in), nb, s, Ns, sL + (size_t)sl * T::SITE_LREALS, slow);
+#pragma unroll
+          for (int c = 0; c < 24; ++c) acc[c] = slow[c];
         }
       }
     } else {
@@ -704,63 +807,18 @@ __global__ void __launch_bounds__(256) k_hop(const HopArgs a) {
           for (int q = 0; q < 12; ++q) upk2(o[q], acc[2 * q], acc[2 * q + 1]);
         }
       } else {
-        // FP64: M5 (or M5^T) along s, Eq. 8, as a recurrence, which halves the FP64
-        // operations that limit these kernels: one 16-byte column (two reals of one
-        // chirality) of one site per item; a closure sweep, then the sweep that overwrites
-        // the column with the result (the item owns its column)
+        // FP64: M5 (or M5^T) along s, Eq. 8, as a recurrence: one 16-byte column (two reals of
+        // one chirality) of one site per item, which owns it
         {
-          constexpr int CW = 2, NCK = 12;
-          using V = double2;
-          const R kap = (R)a.kappa;
+          constexpr int NCK = 12;
           const R *sT = reinterpret_cast<const R *>(sKb);
           for (int item = tid; item < nsite * NCK; item += nthr) {
             const int l = item / NCK, k = item - l * NCK;
             const int chi = k >= NCK / 2 ? 1 : 0;
             const bool bwd = (chi ^ a.mtrans) != 0;
-            const R *Tc = sT + chi * Ns * 8;
-            R *col = sB + (size_t)l * sstride + k * CW;
-            R zc[CW], vl[CW];
-#pragma unroll
-            for (int q = 0; q < CW; ++q) zc[q] = 0;
-#pragma unroll 4
-            for (int j = 0; j < Ns; ++j) {
-              const int sj = bwd ? Ns - 1 - j : j;
-              const V w4 = *reinterpret_cast<const V *>(col + sj * ROW);
-              const R *v = reinterpret_cast<const R *>(&w4);
-              const R w = Tc[j * 8 + 6];
-#pragma unroll
-              for (int q = 0; q < CW; ++q) {
-                zc[q] += w * v[q];
-                vl[q] = v[q];
-              }
-            }
-            R zp[CW], vp[CW];
-#pragma unroll
-            for (int q = 0; q < CW; ++q) {
-              zp[q] = kap * zc[q];
-              vp[q] = kap * vl[q];
-            }
-#pragma unroll 4
-            for (int j = 0; j < Ns; ++j) {
-              const int sj = bwd ? Ns - 1 - j : j;
-              R t[8];
-#pragma unroll
-              for (int e = 0; e < 8; ++e) t[e] = Tc[j * 8 + e];
-              V *cp = reinterpret_cast<V *>(col + sj * ROW);
-              const V w4 = *cp;
-              const R *v = reinterpret_cast<const R *>(&w4);
-              V o4;
-              R *o = reinterpret_cast<R *>(&o4);
-#pragma unroll
-              for (int q = 0; q < CW; ++q) {
-                const R g = t[0] * v[q] + t[1] * vp[q];
-                const R z = (g - t[2] * zp[q]) * t[3];
-                o[q] = t[4] * z + t[5] * zp[q];
-                zp[q] = z;
-                vp[q] = v[q];
-              }
-              *cp = o4;
-            }
+            double2 *col = reinterpret_cast<double2 *>(sB + (size_t)l * sstride + 2 * k) + (bwd ? (Ns - 1) * (ROW / 2) : 0);
+            s_recurrence(col, bwd ? -(ROW / 2) : ROW / 2, sT + chi * Ns * RC_N, Ns, a.kappa,
+                         a.mtrans ? REC_MUL_SOLVE : REC_SOLVE_MUL);
           }
         }
         __syncthreads();

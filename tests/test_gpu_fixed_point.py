@@ -1,0 +1,97 @@
+"""The FP64 hop's fixed-point products (dwf_device.cuh) where the exponents matter: fields whose
+sites differ by many powers of ten, values at the ends of the FP64 range, values that are not
+finite, and links that are not SU(3) (the kernels then take plain FP64 arithmetic).
+
+Tolerance: each output real of D^EO is a sum over eight neighbours of products with links.
+FP64 arithmetic in any order keeps it within 8 * 12 roundings of 2^-53 times the largest
+neighbour (times the link's norm), and the fixed-point form's truncation is below that: 1e-14
+of the largest neighbouring |psi| (about 90 * 1.1e-16), times the largest link row norm.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1101_0423_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+DIMS, NS = (4, 6, 4, 2), 6
+
+
+def neighbour_max(x):
+    """max |psi| over the eight neighbours of each site, per s (shape V4, Ns)."""
+    d = DIMS
+    m = np.abs(x.reshape(d[3], d[2], d[1], d[0], NS, 24)).max(-1)
+    out = np.zeros_like(m)
+    for ax in range(4):
+        out = np.maximum(out, np.maximum(np.roll(m, 1, ax), np.roll(m, -1, ax)))
+    return out.reshape(-1, NS)
+
+
+def run(dwf, U, x):
+    om, sg = inputs.weights("shamir", NS)
+    with dwf.Context(DIMS, NS, 1.8, 0.05, om, sg, U) as ctx:
+        return dwf.dwf_apply_eo(ctx.h, dwf.OP_DEO, dwf.PREC_F64, 0, x).reshape(-1, NS, 24)
+
+
+def check(dwf, U, x, link=1.0):
+    got, want = run(dwf, U, x), oracle.hop(DIMS, NS, U, 0, x).reshape(-1, NS, 24)
+    bound = 1e-14 * link * neighbour_max(x)[..., None] + 5e-324
+    on = inputs.site_parity(DIMS) == 0
+    assert (np.abs(got - want) <= bound)[on].all(), np.max((np.abs(got - want) / bound)[on])
+    assert not got[~on].any()
+
+
+@pytest.mark.parametrize("decades", [0, 3, 30, 250])
+def test_sites_of_different_size(gpu_lib, decades):
+    U = inputs.gauge_field(DIMS, 0.5, seed=51)
+    x = inputs.gaussian_source(DIMS, NS, seed=52).reshape(-1, NS, 24)
+    rng = np.random.RandomState(decades)
+    x = x * 10.0 ** rng.uniform(-decades, decades, size=(x.shape[0], NS, 1))
+    check(gpu_lib, U, np.ascontiguousarray(x).reshape(-1))
+
+
+@pytest.mark.parametrize("scale", [1e-320, 1e-308, 1e-290, 1e-284, 1e150, 1e290, 1e306])
+def test_ends_of_the_range(gpu_lib, scale):
+    U = inputs.gauge_field(DIMS, 0.5, seed=53)
+    x = inputs.gaussian_source(DIMS, NS, seed=54) * scale
+    got, want = run(gpu_lib, U, x), oracle.hop(DIMS, NS, U, 0, x).reshape(-1, NS, 24)
+    bound = 1e-14 * neighbour_max(x)[..., None] + 200 * 5e-324  # denormal results: absolute roundings
+    assert (np.abs(got - want) <= bound).all()
+
+
+def test_links_that_are_not_unitary(gpu_lib):
+    U = inputs.gauge_field(DIMS, 0.5, seed=55).reshape(-1, 18)
+    U[::7] *= 1.003   # inside the checked bound
+    U[3::11] *= 40.0  # outside it
+    U[5::13] *= 1e-5
+    x = inputs.gaussian_source(DIMS, NS, seed=56)
+    check(gpu_lib, U.reshape(-1), x, link=40.0)
+    check(gpu_lib, np.zeros_like(U).reshape(-1), x)
+
+
+def test_values_that_are_not_finite(gpu_lib):
+    """A NaN or an infinity reaches the outputs that its spin projections enter (h_j of Eq. 12
+    for each direction, all colours), and no others: those are as with a zero in its place."""
+    U = inputs.gauge_field(DIMS, 0.5, seed=57)
+    x = inputs.gaussian_source(DIMS, NS, seed=58).reshape(-1, NS, 24)
+    odd = np.flatnonzero(inputs.site_parity(DIMS) == 1)
+    nx, ny, nz, nt = DIMS
+    expect = np.zeros((nt, nz, ny, nx, NS, 4), bool)
+    for site, s, c, v in ((odd[3], 1, 5, np.nan), (odd[40], 4, 17, np.inf), (odd[77], 0, 20, -np.inf)):
+        x[site, s, c] = v
+        at = [site // (nx * ny * nz), site // (nx * ny) % nz, site // nx % ny, site % nx]
+        spin = c // 6
+        for mu in range(4):
+            j = spin if spin < 2 else (1 - (spin - 2) if mu < 2 else spin - 2)
+            for step in (1, -1):
+                to = list(at)
+                to[3 - mu] = (to[3 - mu] + step) % DIMS[mu]
+                expect[tuple(to) + (s, j)] = True
+                expect[tuple(to) + (s, 2 + (1 - j if mu < 2 else j))] = True
+    got = run(gpu_lib, U, x.reshape(-1))
+    bad = np.repeat(expect.reshape(-1, NS, 4), 6, axis=2)
+    assert np.array_equal(~np.isfinite(got), bad)
+    clean = np.where(np.isfinite(x), x, 0.0).reshape(-1)
+    want = oracle.hop(DIMS, NS, U, 0, clean).reshape(-1, NS, 24)
+    bound = 1e-14 * neighbour_max(clean)[..., None]
+    assert (np.abs(got - want) <= bound)[~bad].all()
