@@ -69,9 +69,10 @@ struct dwf_ctx {
   std::vector<double> mat[dwf::MK_COUNT];
   // device matrices per arithmetic precision (0: double, 1: float), kernel order
   void *dmat[2][dwf::MK_COUNT] = {};
-  // M5, M5^T, S1 and S2 as FP64 recurrence tables along s (RC_A); empty where there is none
+  // the same as FP64 recurrence tables along s (RC_A); empty where there is none
   std::vector<double> rec[dwf::MK_COUNT];
   double *drec[dwf::MK_COUNT] = {};
+  bool rec_tight[dwf::MK_COUNT] = {};  // as accurate as the dense matrix: used by s-mixing too
   int *d_nbr[2] = {nullptr, nullptr};
   double *d_U = nullptr;  // FP64 host-layout copy of the gauge field
   void *d_gauge[4][2] = {};

@@ -913,6 +913,9 @@ enum {
 struct SmixArgs {
   Field in, out, out2, r, p, x;
   const void *K, *K2;  // K[chi][t][s]
+  const double *rec, *rec2;  // FP64: the same as recurrence tables (RC_A); rec null: dense
+  double kappa;              // corner of L (Eq. 4)
+  int mtrans, form;          // rec is M5^T (direction of each chirality); REC_* form
   double coef;
   long h;
   int Ns;
@@ -1018,6 +1021,82 @@ __global__ void __launch_bounds__(256) k_smix(const SmixArgs a) {
     store_sp<P>(which == 0 ? F(a.out) : F(a.out2), cb, s, Ns, o);
   }
 }
+
+// FP64 matrices along s as recurrences (S_PLAIN, S_G5, S_CGP; RC_A): four FP64 operations a
+// real against Ns for the dense rows of k_smix, which the FP64 pipe bounded (16^3x32x16: M5^T
+// 693 us dense, 216 us so).  A CTA of (Ns, spb) threads puts its sites' columns (16 bytes x Ns, one
+// pair of reals) into shared memory in coalesced chunks, one thread runs each column, and the
+// result leaves in chunks again.  Columns are an odd number of 16-byte units apart, so that
+// the eight columns of a quarter-warp fall in distinct banks.
+__host__ __device__ inline int srec_stride(int Ns) { return Ns | 1; }
+__host__ __device__ inline size_t srec_smem_bytes(int spb, int Ns) {
+  return (size_t)spb * 12 * srec_stride(Ns) * 16 + (size_t)2 * Ns * RC_N * 8;
+}
+template <int MODE>
+__global__ void __launch_bounds__(256) k_srec(const SmixArgs a) {
+  const int rb = blockIdx.y;
+  auto F = [&](const Field &f) { return rb ? field_rhs(f, rb, a.fstride, a.nstride) : f; };
+  CGScalars *const sc_ = a.sc + rb;
+  extern __shared__ __align__(128) unsigned char sm[];
+  const int Ns = a.Ns, cs = srec_stride(Ns);
+  const int s = threadIdx.x, sl = threadIdx.y, spb = blockDim.y;
+  const int tid = s + sl * Ns, nthr = Ns * spb;
+  const long cb0 = (long)blockIdx.x * spb, cb = cb0 + sl;
+  const bool active = cb < a.h;
+  if (a.use_flag && sc_->restart_flag) return;
+  double2 *sV = reinterpret_cast<double2 *>(sm);
+  double *sT = reinterpret_cast<double *>(sV + (size_t)spb * 12 * cs);
+  for (int i = tid; i < 2 * Ns * RC_N; i += nthr) {
+    const int e = i % RC_N;
+    sT[i] = (e == RC_A || e == RC_B || e == RC_W) ? a.coef * a.rec[i] : a.rec[i];
+  }
+  const size_t base = (size_t)cb * 12 * Ns + s;  // chunk k at base + k Ns
+  double2 *mine = sV + (size_t)sl * 12 * cs + s;
+  if (active) {
+    if constexpr (MODE == S_CGP) {
+      // x += alpha p (the previous step), p = r + beta p (as k_smix)
+      const double alpha = sc_->alpha, beta = sc_->beta;
+      const Field fx = rb ? field_rhs(a.x, rb, a.xfstride, 0) : a.x;
+      double2 *gp = static_cast<double2 *>(F(a.p).v) + base, *gx = static_cast<double2 *>(fx.v) + base;
+      const double2 *gr = static_cast<const double2 *>(F(a.r).v) + base;
+#pragma unroll 4
+      for (int k = 0; k < 12; ++k) {
+        double2 p = gp[k * Ns], x = gx[k * Ns];
+        const double2 r = gr[k * Ns];
+        x.x += alpha * p.x, x.y += alpha * p.y;
+        gx[k * Ns] = x;
+        p.x = r.x + beta * p.x, p.y = r.y + beta * p.y;
+        gp[k * Ns] = p;
+        mine[k * cs] = k < 6 ? p : make_double2(-p.x, -p.y);
+      }
+    } else {
+      const double2 *gi = static_cast<const double2 *>(F(a.in).v) + base;
+#pragma unroll
+      for (int k = 0; k < 12; ++k) {
+        const double2 v = __ldg(gi + k * Ns);
+        mine[k * cs] = MODE == S_G5 && k >= 6 ? make_double2(-v.x, -v.y) : v;
+      }
+    }
+  }
+  __syncthreads();
+  const int ncol = (int)min((long)spb, a.h - cb0) * 12;
+  for (int col = tid; col < ncol; col += nthr) {
+    const int chi = col % 12 >= 6 ? 1 : 0;
+    const bool bwd = (chi ^ a.mtrans) != 0;
+    s_recurrence(sV + (size_t)col * cs + (bwd ? Ns - 1 : 0), bwd ? -1 : 1, sT + chi * Ns * RC_N, Ns, a.kappa, a.form);
+  }
+  __syncthreads();
+  if (active) {
+    double2 *go = static_cast<double2 *>(F(a.out).v) + base;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) go[k * Ns] = mine[k * cs];
+  }
+}
+
+// FP64 S_DUAL with two cyclic bidiagonal matrices (omega + sigma L and (d - m0)(omega + sigma L)
+// + 1 - L of Eq. 5, or 1 and d - m0): tables of RC_A with the diagonal in A and the factor of L
+// in B.  Two multiply-adds a real and matrix; each slice reads its neighbour along s through L1.
+__global__ void __launch_bounds__(256) k_sdual(const SmixArgs a);
 
 // ------------------------------------------------------------------ per-(site, s) vector kernels
 
@@ -1202,6 +1281,36 @@ __global__ void k_gauge(const double *U, typename PT<P>::lreal *G, Geom g, int p
 }
 
 #ifdef DWF_DEFINE_PLAIN_KERNELS  // non-template kernels: defined in one translation unit only
+
+__global__ void __launch_bounds__(256) k_sdual(const SmixArgs a) {
+  const int Ns = a.Ns, s = threadIdx.x;
+  const long cb = (long)blockIdx.x * blockDim.y + threadIdx.y;
+  if (cb >= a.h) return;
+  const double2 *gi = static_cast<const double2 *>(a.in.v) + (size_t)cb * 12 * Ns;
+  double2 *g1 = static_cast<double2 *>(a.out.v) + (size_t)cb * 12 * Ns + s;
+  double2 *g2 = static_cast<double2 *>(a.out2.v) + (size_t)cb * 12 * Ns + s;
+#pragma unroll
+  for (int chi = 0; chi < 2; ++chi) {
+    const int j = chi ? Ns - 1 - s : s;                                // step of this slice
+    const int sn = chi ? (s + 1 < Ns ? s + 1 : 0) : (s ? s : Ns) - 1;  // (L v)_s reads v at sn
+    const double *T1 = a.rec + (chi * Ns + j) * RC_N, *T2 = a.rec2 + (chi * Ns + j) * RC_N;
+    const double kc = j ? a.coef : a.coef * a.kappa;
+    const double d1 = a.coef * T1[RC_A], o1 = kc * T1[RC_B], d2 = a.coef * T2[RC_A], o2 = kc * T2[RC_B];
+    const bool b1 = o1 != 0.0, b2 = o2 != 0.0;
+#pragma unroll
+    for (int k = 6 * chi; k < 6 * chi + 6; ++k) {
+      const double2 v = __ldg(gi + k * Ns + s);
+      double2 u1 = make_double2(d1 * v.x, d1 * v.y), u2 = make_double2(d2 * v.x, d2 * v.y);
+      if (b1 || b2) {
+        const double2 w = __ldg(gi + k * Ns + sn);
+        if (b1) u1 = make_double2(fma(o1, w.x, u1.x), fma(o1, w.y, u1.y));
+        if (b2) u2 = make_double2(fma(o2, w.x, u2.x), fma(o2, w.y, u2.y));
+      }
+      g1[k * Ns] = u1;
+      g2[k * Ns] = u2;
+    }
+  }
+}
 
 // |a - b|^2 (both FP64) -> fin
 __global__ void __launch_bounds__(256) k_diff_norm2(const VecArgs v) {

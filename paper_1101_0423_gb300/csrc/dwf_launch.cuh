@@ -147,13 +147,47 @@ cudaError_t smix_go(const SmixArgs &a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+// FP64 recurrences: CTAs of about 128 threads, so that several share an SM and one's loads
+// overlap another's FP64 phase
+template <int MODE>
+cudaError_t srec_go(const SmixArgs &a, cudaStream_t st) {
+  const int spb = sites_per_block(P_F64, a.Ns);
+  const size_t smem = srec_smem_bytes(spb, a.Ns);
+  if (smem > 48 * 1024) {
+    static std::mutex cmu;
+    static size_t configured = 0;
+    std::lock_guard<std::mutex> lock(cmu);
+    if (configured < smem) {
+      cudaError_t e = cudaFuncSetAttribute(k_srec<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+      configured = smem;
+    }
+  }
+  const long nblk = (a.h + spb - 1) / spb;
+  k_srec<MODE><<<dim3((unsigned)nblk, a.nrhs > 1 ? a.nrhs : 1), dim3(a.Ns, spb), smem, st>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t sdual_launch(const SmixArgs &a, cudaStream_t st);
+
 template <int P>
 cudaError_t smix_launch(int mode, const SmixArgs &a, cudaStream_t st) {
-  switch (mode) {
-    case S_PLAIN: return smix_go<P, S_PLAIN>(a, st);
-    case S_G5: return smix_go<P, S_G5>(a, st);
-    case S_CGP: return smix_go<P, S_CGP>(a, st);
-    case S_DUAL: return smix_go<P, S_DUAL>(a, st);
+  if constexpr (P == P_F64) {
+    // as recurrences; dense only where a matrix has no table as accurate as its rows (16^3x32x16:
+    // 216 us against 693 us)
+    switch (mode) {
+      case S_PLAIN: return a.rec ? srec_go<S_PLAIN>(a, st) : smix_go<P, S_PLAIN>(a, st);
+      case S_G5: return a.rec ? srec_go<S_G5>(a, st) : smix_go<P, S_G5>(a, st);
+      case S_CGP: return a.rec ? srec_go<S_CGP>(a, st) : smix_go<P, S_CGP>(a, st);
+      case S_DUAL: return sdual_launch(a, st);
+    }
+  } else {
+    switch (mode) {
+      case S_PLAIN: return smix_go<P, S_PLAIN>(a, st);
+      case S_G5: return smix_go<P, S_G5>(a, st);
+      case S_CGP: return smix_go<P, S_CGP>(a, st);
+      case S_DUAL: return smix_go<P, S_DUAL>(a, st);
+    }
   }
   return cudaErrorInvalidValue;
 }

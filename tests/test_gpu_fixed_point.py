@@ -95,3 +95,28 @@ def test_values_that_are_not_finite(gpu_lib):
     want = oracle.hop(DIMS, NS, U, 0, clean).reshape(-1, NS, 24)
     bound = 1e-14 * neighbour_max(clean)[..., None]
     assert (np.abs(got - want) <= bound)[~bad].all()
+
+
+@pytest.mark.parametrize("opname", ["M5", "M5T", "DFULL"])
+@pytest.mark.parametrize("ns,ratio", [(1, 1.0), (2, 0.0), (7, 1.0), (16, 1.0), (33, 0.5), (64, 1.0), (16, 1.8), (32, 1.8)])
+def test_matrices_along_s(gpu_lib, opname, ns, ratio):
+    """The FP64 s-mixing kernel as a recurrence and, where sigma > omega makes the recurrence
+    grow along s, dense: each output is a sum of Ns products, so 1e-14 (about 45 * 2 eps) of the
+    field's size times the matrix's.  The reference matrix is M5 = P A^{-1} with the cyclic
+    bidiagonal A = (d - m0) P + omega^{-1/2} (1 - L), P = sqrt(omega) (1 + cL): A's condition
+    number is below 60 for these weights, that of 1 + cL (which Eq. 8 inverts) up to 1.8^32."""
+    dwf, dims, mq = gpu_lib, (2, 4, 2, 6), 0.05
+    om, sg = np.ones(ns), ratio * np.ones(ns)
+    U = inputs.gauge_field(dims, 0.5, seed=60)
+    x = inputs.gaussian_source(dims, ns, seed=61)
+    L = np.diag(np.ones(ns - 1), -1)
+    L[0, -1] += -mq / (2 * 1.8)
+    P = [np.diag(np.sqrt(om)) @ (np.eye(ns) + np.diag(sg / om) @ l) for l in (L, L.T)]
+    mp, mm = [p @ np.linalg.inv(2.2 * p + np.diag(1 / np.sqrt(om)) @ (np.eye(ns) - l)) for p, l in zip(P, (L, L.T))]
+    with dwf.Context(dims, ns, 1.8, mq, om, sg, U) as ctx:
+        got = dwf.dwf_apply_eo(ctx.h, getattr(dwf, "OP_" + opname), dwf.PREC_F64, 1, x)
+    if opname == "DFULL":
+        want = oracle.dfull(dims, ns, U, 1.8, mq, om, sg, x)
+    else:
+        want = oracle.apply_s(dims, ns, mp, mm, x, transpose=opname == "M5T", parity=1)
+    assert np.abs(got - want).max() <= 1e-14 * max(1.0, np.abs(want).max())
