@@ -459,21 +459,22 @@ cudaError_t accum_any(int prec, const VecArgs &v, int sm, cudaStream_t st) {
   }
   return cudaErrorInvalidValue;
 }
-cudaError_t pack_any(int prec, const double *host, Field f, Geom g, int par, int sm, cudaStream_t st) {
+cudaError_t pack_any(int prec, const double *host, Field f, Geom g, int par, cudaStream_t st) {
   switch (prec) {
-    case P_F64: return pack_launch<P_F64>(host, f, g, par, sm, st);
-    case P_F32: return pack_launch<P_F32>(host, f, g, par, sm, st);
-    case P_F16: return pack_launch<P_F16>(host, f, g, par, sm, st);
-    case P_BF16: return pack_launch<P_BF16>(host, f, g, par, sm, st);
+    case P_F64: return pack_launch<P_F64>(host, f, g, par, st);
+    case P_F32: return pack_launch<P_F32>(host, f, g, par, st);
+    case P_F16: return pack_launch<P_F16>(host, f, g, par, st);
+    case P_BF16: return pack_launch<P_BF16>(host, f, g, par, st);
   }
   return cudaErrorInvalidValue;
 }
-cudaError_t unpack_any(int prec, Field f, double *host, Geom g, int par, int sm, cudaStream_t st) {
+// zero_other: the sites of the other parity are set to 0 in the same pass
+cudaError_t unpack_any(int prec, Field f, double *host, Geom g, int par, bool zero_other, cudaStream_t st) {
   switch (prec) {
-    case P_F64: return unpack_launch<P_F64>(f, host, g, par, sm, st);
-    case P_F32: return unpack_launch<P_F32>(f, host, g, par, sm, st);
-    case P_F16: return unpack_launch<P_F16>(f, host, g, par, sm, st);
-    case P_BF16: return unpack_launch<P_BF16>(f, host, g, par, sm, st);
+    case P_F64: return unpack_launch<P_F64>(f, host, g, par, zero_other, st);
+    case P_F32: return unpack_launch<P_F32>(f, host, g, par, zero_other, st);
+    case P_F16: return unpack_launch<P_F16>(f, host, g, par, zero_other, st);
+    case P_BF16: return unpack_launch<P_BF16>(f, host, g, par, zero_other, st);
   }
   return cudaErrorInvalidValue;
 }
@@ -1083,7 +1084,6 @@ dwf_status dwf_apply_eo_dev(dwf_ctx *c, int op, int prec, int parity, const doub
   TRY(ensure_gauge(c, prec, st));
   const Geom g = geom(c);
   const int cls = DWF_KC_OTHER;
-  CK(cudaMemsetAsync(d_out, 0, full, st));
 
   Field in[2], out[2], tA, tB, tC;
   for (int p = 0; p < 2; ++p) {
@@ -1095,12 +1095,12 @@ dwf_status dwf_apply_eo_dev(dwf_ctx *c, int op, int prec, int parity, const doub
   TRY(get_buf(c, "ap_tC", prec, &tC));
   auto pack = [&](int p) -> dwf_status {
     Timed t(c, st, cls);
-    CK(pack_any(prec, d_in, in[p], g, p, c->sm_count, st));
+    CK(pack_any(prec, d_in, in[p], g, p, st));
     return DWF_OK;
   };
   auto unpack = [&](int p) -> dwf_status {
     Timed t(c, st, cls);
-    CK(unpack_any(prec, out[p], d_out, g, p, c->sm_count, st));
+    CK(unpack_any(prec, out[p], d_out, g, p, op != DWF_OP_DFULL && op != DWF_OP_DW, st));
     return DWF_OK;
   };
   switch (op) {
@@ -1538,7 +1538,7 @@ struct SolveRun {
     for (int p = 0; p < 2; ++p) {
       {
         Timed t(c, st, DWF_KC_F64);
-        CK(pack_any(P_F64, d_rhs + (size_t)k * full_doubles, eta[p], g, p, c->sm_count, st));
+        CK(pack_any(P_F64, d_rhs + (size_t)k * full_doubles, eta[p], g, p, st));
       }
       TRY(smix(c, st, P_F64, S_PLAIN, eta[p], etap[p], MK_S1, 1.0, DWF_KC_F64));
     }
@@ -1646,7 +1646,7 @@ struct SolveRun {
         TRY(hop(c, st, P_F64, E_M_XPAY, a, DWF_KC_F64));
       } else {
         Timed t(c, st, DWF_KC_F64);
-        CK(pack_any(P_F64, d_rhs + (size_t)k * full_doubles, bk, g, S.sp, c->sm_count, st));
+        CK(pack_any(P_F64, d_rhs + (size_t)k * full_doubles, bk, g, S.sp, st));
       }
       TRY(norm2(c, st, P_F64, bk, FIN_RED));
       CK(cudaMemcpyAsync(at(c, S.rh, k, P_F64).v, bk.v, nbytes64, cudaMemcpyDeviceToDevice, st));
@@ -1797,7 +1797,7 @@ struct SolveRun {
     for (int p = 0; p < 2; ++p) {
       TRY(smix(c, st, P_F64, S_PLAIN, phi[p], psi[p], MK_S2, 1.0, DWF_KC_F64));
       Timed t(c, st, DWF_KC_F64);
-      CK(unpack_any(P_F64, psi[p], d_sol + (size_t)k * full_doubles, g, p, c->sm_count, st));
+      CK(unpack_any(P_F64, psi[p], d_sol + (size_t)k * full_doubles, g, p, false, st));
     }
     TRY(op_full(c, st, P_F64, psi, dpsi, MK_W, MK_Z, DWF_KC_F64));
     double num = 0, den = 0;
@@ -1847,10 +1847,9 @@ struct SolveRun {
         for (int k : again) TRY(reconstruct(k));
       }
     } else {
-      CK(cudaMemsetAsync(d_sol, 0, (size_t)K * full_doubles * sizeof(double), st));
       for (int k = 0; k < K; ++k) {
         Timed t(c, st, DWF_KC_F64);
-        CK(unpack_any(P_F64, at(c, S.xh, k, P_F64), d_sol + (size_t)k * full_doubles, g, S.sp, c->sm_count, st));
+        CK(unpack_any(P_F64, at(c, S.xh, k, P_F64), d_sol + (size_t)k * full_doubles, g, S.sp, true, st));
       }
     }
     ++pass;
@@ -2377,7 +2376,6 @@ extern "C" dwf_status dwf_apply_eo_dev_static(dwf_ctx *c, int op, int prec, int 
   // ticket must start at zero
   CK(cudaMemsetAsync(sc, 0, sizeof(CGScalars), st));
   CK(cudaMemsetAsync(ticket, 0, sizeof(unsigned), st));
-  CK(cudaMemsetAsync(d_out, 0, full, st));
   const Geom g = geom(c);
   Field &in = f[0], &out = f[1], &tA = f[2], &tB = f[3], &tC = f[4];
   const int inpar = op == DWF_OP_DEO ? 1 : op == DWF_OP_DOE ? 0 : parity;
@@ -2417,7 +2415,7 @@ extern "C" dwf_status dwf_apply_eo_dev_static(dwf_ctx *c, int op, int prec, int 
     if (e == cudaSuccess) e = hop_s(sp, E_XPAY_G5, t, v, q, false, false, 0.5);
     return e;
   };
-  CK(pack_any(prec, d_in, in, g, inpar, c->sm_count, st));
+  CK(pack_any(prec, d_in, in, g, inpar, st));
   switch (op) {
     case DWF_OP_DEO:
     case DWF_OP_DOE:
@@ -2438,7 +2436,7 @@ extern "C" dwf_status dwf_apply_eo_dev_static(dwf_ctx *c, int op, int prec, int 
       CK(apply_c(parity, tC, out, tA));
       break;
   }
-  CK(unpack_any(prec, out, d_out, g, outpar, c->sm_count, st));
+  CK(unpack_any(prec, out, d_out, g, outpar, true, st));
   // the call returns when its work is done: it waits for `stream` and reads the kernels'
   // error word (a bounded device-side wait that gave up) into host memory of its own
   int err = 0;
@@ -2722,7 +2720,7 @@ dwf_status part_scatter_local(dwf_ctx *c, const double *in, const std::string &n
   CK(cudaMemcpyAsync(d, in, n * sizeof(double), cudaMemcpyHostToDevice, c->stream));
   Field f;
   TRY(part_field(c, name, prec, &f));
-  CK(pack_any(prec, static_cast<const double *>(d), f, local_geom(c->pg, c->Ns), p, c->sm_count, c->stream));
+  CK(pack_any(prec, static_cast<const double *>(d), f, local_geom(c->pg, c->Ns), p, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   return DWF_OK;
 }
@@ -2733,7 +2731,7 @@ dwf_status part_gather_local(dwf_ctx *c, const std::string &name, int prec, int 
   CK(cudaMemcpyAsync(d, out, n * sizeof(double), cudaMemcpyHostToDevice, c->stream));
   Field f;
   TRY(part_field(c, name, prec, &f));
-  CK(unpack_any(prec, f, static_cast<double *>(d), local_geom(c->pg, c->Ns), p, c->sm_count, c->stream));
+  CK(unpack_any(prec, f, static_cast<double *>(d), local_geom(c->pg, c->Ns), p, false, c->stream));
   CK(cudaMemcpyAsync(out, d, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   return DWF_OK;
@@ -2770,7 +2768,7 @@ dwf_status part_scatter(const PartSet &ps, const double *g_in, const std::string
     CK(cudaMemcpyAsync(d, buf.data(), buf.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream));
     Field f;
     TRY(part_field(c, name, prec, &f));
-    CK(pack_any(prec, static_cast<const double *>(d), f, local_geom(g, c->Ns), p, c->sm_count, c->stream));
+    CK(pack_any(prec, static_cast<const double *>(d), f, local_geom(g, c->Ns), p, c->stream));
     CK(cudaStreamSynchronize(c->stream));
   }
   return DWF_OK;
@@ -2788,7 +2786,7 @@ dwf_status part_gather(const PartSet &ps, const std::string &name, int prec, int
     CK(cudaMemsetAsync(d, 0, (size_t)2 * g.h * gsite * sizeof(double), c->stream));
     Field f;
     TRY(part_field(c, name, prec, &f));
-    CK(unpack_any(prec, f, static_cast<double *>(d), local_geom(g, c->Ns), p, c->sm_count, c->stream));
+    CK(unpack_any(prec, f, static_cast<double *>(d), local_geom(g, c->Ns), p, false, c->stream));
     buf.assign((size_t)2 * g.h * gsite, 0.0);
     CK(cudaMemcpyAsync(buf.data(), d, buf.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));

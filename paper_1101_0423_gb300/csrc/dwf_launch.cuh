@@ -218,14 +218,17 @@ cudaError_t accum_launch(const VecArgs &v, int sm_count, cudaStream_t st) {
 }
 
 template <int P>
-cudaError_t pack_launch(const double *host, Field out, Geom g, int parity, int sm_count, cudaStream_t st) {
-  k_pack<P><<<vec_grid(g.h * g.Ns, sm_count), 256, 0, st>>>(host, out, g, parity);
+cudaError_t pack_launch(const double *host, Field out, Geom g, int parity, cudaStream_t st) {
+  const int spb = sites_per_block(P_F64, g.Ns);
+  k_pack<P><<<(unsigned)((g.h + spb - 1) / spb), dim3(g.Ns, spb), host_stage_bytes(spb, g.Ns), st>>>(host, out, g, parity);
   return cudaGetLastError();
 }
 
 template <int P>
-cudaError_t unpack_launch(Field in, double *host, Geom g, int parity, int sm_count, cudaStream_t st) {
-  k_unpack<P><<<vec_grid(g.h * g.Ns, sm_count), 256, 0, st>>>(in, host, g, parity);
+cudaError_t unpack_launch(Field in, double *host, Geom g, int parity, int zero_other, cudaStream_t st) {
+  const int spb = sites_per_block(P_F64, g.Ns);
+  k_unpack<P><<<(unsigned)((g.h + spb - 1) / spb), dim3(g.Ns, spb), host_stage_bytes(spb, g.Ns), st>>>(in, host, g, parity,
+                                                                                                    zero_other);
   return cudaGetLastError();
 }
 
@@ -243,7 +246,7 @@ cudaError_t gauge_launch(const double *U, void *G, Geom g, int parity, int sm_co
   extern template cudaError_t norm2_launch<P>(const VecArgs &, int, cudaStream_t);                   \
   extern template cudaError_t convert_launch<P>(int, const VecArgs &, int, cudaStream_t);            \
   extern template cudaError_t accum_launch<P>(const VecArgs &, int, cudaStream_t);                   \
-  extern template cudaError_t pack_launch<P>(const double *, Field, Geom, int, int, cudaStream_t);    \
+  extern template cudaError_t pack_launch<P>(const double *, Field, Geom, int, cudaStream_t);         \
   extern template cudaError_t unpack_launch<P>(Field, double *, Geom, int, int, cudaStream_t);       \
   extern template cudaError_t gauge_launch<P>(const double *, void *, Geom, int, int, cudaStream_t);
 
@@ -253,7 +256,7 @@ cudaError_t gauge_launch(const double *U, void *G, Geom g, int parity, int sm_co
   template cudaError_t norm2_launch<P>(const VecArgs &, int, cudaStream_t);                   \
   template cudaError_t convert_launch<P>(int, const VecArgs &, int, cudaStream_t);            \
   template cudaError_t accum_launch<P>(const VecArgs &, int, cudaStream_t);                   \
-  template cudaError_t pack_launch<P>(const double *, Field, Geom, int, int, cudaStream_t);    \
+  template cudaError_t pack_launch<P>(const double *, Field, Geom, int, cudaStream_t);         \
   template cudaError_t unpack_launch<P>(Field, double *, Geom, int, int, cudaStream_t);       \
   template cudaError_t gauge_launch<P>(const double *, void *, Geom, int, int, cudaStream_t);
 
