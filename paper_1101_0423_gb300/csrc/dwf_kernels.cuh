@@ -400,7 +400,7 @@ __device__ __noinline__ void hop_site_f64(const Field in, const int *nb, int s, 
 // phase (C C^dag in FP64 at 16^3x32x16: 3.83 ms, against 4.05 ms with three CTAs of 168
 // registers, and 11.0 ms with the products in FP64).
 template <int P, int EPI, int NSC>
-__global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 1) k_hop(const HopArgs a) {
+__global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_hop(const HopArgs a) {
   // one right-hand side of a batch per grid row; fields are offset where they are used, so
   // the pointers stay in parameter space instead of registers
   const int rb = blockIdx.y;
