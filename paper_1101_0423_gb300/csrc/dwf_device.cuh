@@ -401,14 +401,13 @@ __device__ __forceinline__ void to_fixed(double x, int E, int &hi, int &lo) {
   lo = (int)(m & 0x3fffffffu) * sg;
 }
 
-__device__ __forceinline__ long long mul_w(int a, int b) { return (long long)a * b; }
-__device__ __forceinline__ void mad_w(long long &c, int a, int b) {
-  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(c) : "r"(a), "r"(b));
-}
+// c + a b, the full 64-bit product
+__device__ __forceinline__ long long mad_w(int a, int b, long long c) { return (long long)a * b + c; }
 
-// h_j = psi_up + S A psi_dn of direction MU (spin projection), FP64
-template <int MU, int S>
-__device__ __forceinline__ void project_f64(const double (&ps)[24], double (&h)[12]) {
+// h_j = psi_up + S A psi_dn of direction MU (spin projection), FP64; one multiply-add a real (the
+// FP64 pipe issues DFMA faster than DADD, and a product with +-1 is exact)
+template <int MU>
+__device__ __forceinline__ void project_f64(const double (&ps)[24], double S, double (&h)[12]) {
 #pragma unroll
   for (int j = 0; j < 2; ++j)
 #pragma unroll
@@ -417,29 +416,30 @@ __device__ __forceinline__ void project_f64(const double (&ps)[24], double (&h)[
       // phase code 0: 1, 1: i, 2: -1, 3: -i
       const int p = a_ph(MU, j);
       const double vr = (p & 1) ? ps[src + 1] : ps[src], vi = (p & 1) ? ps[src] : ps[src + 1];
-      h[dst] = (p == 1 || p == 2) == (S > 0) ? ps[dst] - vr : ps[dst] + vr;
-      h[dst + 1] = (p == 2 || p == 3) == (S > 0) ? ps[dst + 1] - vi : ps[dst + 1] + vi;
+      h[dst] = fma((p == 1 || p == 2) ? -S : S, vr, ps[dst]);
+      h[dst + 1] = fma((p == 2 || p == 3) ? -S : S, vi, ps[dst + 1]);
     }
 }
 
 // acc += (1 + S g_MU) W psi in units of 2^(E - 1080); W: the link's nine entries; returns
 // false if a value is outside the fixed-point range (acc is then meaningless)
-template <int MU, int S>
-__device__ __forceinline__ bool hop_dir_fixed(long long (&acc)[24], int &E, const double (&ps)[24], const int4 *W) {
+template <int MU>
+__device__ __forceinline__ bool hop_dir_fixed(long long (&acc)[24], int &E, const double (&ps)[24], const int4 *W,
+                                              const bool back) {
   double h[12];
-  project_f64<MU, S>(ps, h);
+  project_f64<MU>(ps, back ? 1.0 : -1.0, h);
   int em = 0;
 #pragma unroll
   for (int q = 0; q < 12; ++q) em = max(em, __double2hiint(h[q]) & 0x7fffffff);
   em >>= 20;
   bool ok = em <= FX_EMAX;
-  if (em < FX_EMIN) {  // all zero (nothing to add), or too small for the fixed-point range
+  if (__builtin_expect(em < FX_EMIN, 0)) {  // all zero (nothing to add), or too small for the fixed-point range
     unsigned any = 0;
 #pragma unroll
     for (int q = 0; q < 12; ++q) any |= (unsigned)(__double2hiint(h[q]) << 1) | (unsigned)__double2loint(h[q]);
     ok = any == 0;
   }
-  if (em > E) {
+  if (__builtin_expect(em > E, 0)) {
     const int d = min(em + 1 - E, 63);
 #pragma unroll
     for (int c = 0; c < 24; ++c) acc[c] >>= d;
@@ -455,18 +455,17 @@ __device__ __forceinline__ bool hop_dir_fixed(long long (&acc)[24], int &E, cons
   }
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const int4 w0 = W[3 * a], w1 = W[3 * a + 1], w2 = W[3 * a + 2];
+    const int4 w[3] = {W[3 * a], W[3 * a + 1], W[3 * a + 2]};
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       long long Hr = 0, Hi = 0, Xr = 1 << 29, Xi = 1 << 29;
 #pragma unroll
       for (int b = 0; b < 3; ++b) {
-        const int4 w = b == 0 ? w0 : b == 1 ? w1 : w2;
         const int q = 3 * j + b;
-        mad_w(Hr, w.x, ph[q]), mad_w(Hr, w.z, nh[q]);
-        mad_w(Hi, w.x, qh[q]), mad_w(Hi, w.z, ph[q]);
-        mad_w(Xr, w.x, pl[q]), mad_w(Xr, w.y, ph[q]), mad_w(Xr, w.z, nl[q]), mad_w(Xr, w.w, nh[q]);
-        mad_w(Xi, w.x, ql[q]), mad_w(Xi, w.y, qh[q]), mad_w(Xi, w.z, pl[q]), mad_w(Xi, w.w, ph[q]);
+        Hr = mad_w(w[b].z, nh[q], mad_w(w[b].x, ph[q], Hr));
+        Hi = mad_w(w[b].z, ph[q], mad_w(w[b].x, qh[q], Hi));
+        Xr = mad_w(w[b].w, nh[q], mad_w(w[b].z, nl[q], mad_w(w[b].y, ph[q], mad_w(w[b].x, pl[q], Xr))));
+        Xi = mad_w(w[b].w, ph[q], mad_w(w[b].z, pl[q], mad_w(w[b].y, qh[q], mad_w(w[b].x, ql[q], Xi))));
       }
       const long long re = Hr + (Xr >> 30), im = Hi + (Xi >> 30);
       const int u = 2 * (a + 3 * j);
@@ -477,14 +476,27 @@ __device__ __forceinline__ bool hop_dir_fixed(long long (&acc)[24], int &E, cons
         if (ad_col(MU, k) != j) continue;
         const int dn = 2 * (a + 3 * (2 + k)), p = ad_ph(MU, k);
         // S phase (re + i im): phase 0: 1, 1: i, 2: -1, 3: -i
-        const bool neg_r = (p == 1 || p == 2) == (S > 0), neg_i = (p == 2 || p == 3) == (S > 0);
         const long long vr = (p & 1) ? im : re, vi = (p & 1) ? re : im;
-        acc[dn] = neg_r ? acc[dn] - vr : acc[dn] + vr;
-        acc[dn + 1] = neg_i ? acc[dn + 1] - vi : acc[dn + 1] + vi;
+        acc[dn] = (p == 1 || p == 2) == back ? acc[dn] - vr : acc[dn] + vr;
+        acc[dn + 1] = (p == 2 || p == 3) == back ? acc[dn + 1] - vi : acc[dn + 1] + vi;
       }
     }
   }
   return ok;
+}
+
+// a 2^(k - 1023), rounded to nearest even: as (double)a times a power of two, without the two
+// instructions on the FP64 pipe (C C^dag in FP64 at 16^3x32x16: 2.98 -> 2.83 ms)
+__device__ __forceinline__ double from_fixed(long long a, int k) {
+  const unsigned long long u = a < 0 ? -(unsigned long long)a : (unsigned long long)a;
+  const int z = __clzll((long long)u);
+  const unsigned long long n = u << (z & 63);  // leading one at bit 63
+  // 53 bits with their exponent, and the rest rounded (a carry moves into the exponent)
+  unsigned long long r = (n >> 11) + ((unsigned long long)(k + 62 - z) << 52);
+  const unsigned rest = (unsigned)n & 0x7ffu;
+  r += (rest + 0x3ffu + (unsigned)(r & 1)) >> 11;
+  r |= (unsigned long long)a & 0x8000000000000000ull;
+  return u ? __longlong_as_double((long long)r) : 0.0;
 }
 
 // a link row (three complex entries) in units of 2^-60, split as above; false if its 2-norm is

@@ -397,8 +397,9 @@ __device__ __noinline__ void hop_site_f64(const Field in, const int *nb, int s, 
 // FP64 fixed point, the epilogue.  The FP64
 // forms (fixed-point products, FP64 projections and M5) are capped at 128 registers, four CTAs
 // per SM: a CTA's M5 phase keeps the FP64 pipe busy while others are in their integer hop
-// phase (C C^dag in FP64 at 16^3x32x16: 3.83 ms, against 4.05 ms with three CTAs of 168
-// registers, and 11.0 ms with the products in FP64).
+// phase (C C^dag in FP64 at 16^3x32x16: 11.0 ms with the products in FP64, now 2.8 ms, 5 %
+// less than with three CTAs of 168 registers).  They wait as much on the FP64 pipe's latency
+// (57 % busy) as on issue (33 %): 16 warps per SM.
 template <int P, int EPI, int NSC>
 __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_hop(const HopArgs a) {
   // one right-hand side of a batch per grid row; fields are offset where they are used, so
@@ -605,25 +606,23 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
         bool ok = !slow_tile;
         const int4 *myW = reinterpret_cast<const int4 *>(sP) + (size_t)sl * FX_SITE_I4;
 #pragma unroll
-        for (int d = 0; d < 8; ++d) {
-          R ps[24];
-          load_sp_ro<P>(F(a.in), nb[d], s, Ns, ps);
-          const int4 *W = myW + 9 * d;
-          switch (d) {
-            case 0: ok &= hop_dir_fixed<0, -1>(ai, ex, ps, W); break;
-            case 1: ok &= hop_dir_fixed<1, -1>(ai, ex, ps, W); break;
-            case 2: ok &= hop_dir_fixed<2, -1>(ai, ex, ps, W); break;
-            case 3: ok &= hop_dir_fixed<3, -1>(ai, ex, ps, W); break;
-            case 4: ok &= hop_dir_fixed<0, 1>(ai, ex, ps, W); break;
-            case 5: ok &= hop_dir_fixed<1, 1>(ai, ex, ps, W); break;
-            case 6: ok &= hop_dir_fixed<2, 1>(ai, ex, ps, W); break;
-            default: ok &= hop_dir_fixed<3, 1>(ai, ex, ps, W); break;
+        for (int mu = 0; mu < 4; ++mu) {
+#pragma unroll
+          for (int back = 0; back < 2; ++back) {
+            R ps[24];
+            load_sp_ro<P>(F(a.in), nb[mu + 4 * back], s, Ns, ps);
+            const int4 *W = myW + 9 * (mu + 4 * back);
+            switch (mu) {
+              case 0: ok &= hop_dir_fixed<0>(ai, ex, ps, W, back); break;
+              case 1: ok &= hop_dir_fixed<1>(ai, ex, ps, W, back); break;
+              case 2: ok &= hop_dir_fixed<2>(ai, ex, ps, W, back); break;
+              default: ok &= hop_dir_fixed<3>(ai, ex, ps, W, back); break;
+            }
           }
         }
         if (ok) {
-          const R scale = __hiloint2double((ex - 57) << 20, 0);  // 2^(ex - 1080)
 #pragma unroll
-          for (int c = 0; c < 24; ++c) acc[c] = (R)ai[c] * scale;
+          for (int c = 0; c < 24; ++c) acc[c] = from_fixed(ai[c], ex - 57);  // times 2^(ex - 1080)
         } else {
           R slow[24];
           hop_site_f64<P>(F(a.in), nb, s, Ns, sL + (size_t)sl * T::SITE_LREALS, slow);
@@ -837,22 +836,51 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
       } else if constexpr (EPI == E_M) {
         store_sp<P>(F(a.out), cb, s, Ns, acc);
       } else if constexpr (EPI == E_XPAY_G5 || EPI == E_XPAY) {
-        R y[24];
-        load_sp<P>(F(a.y), cb, s, Ns, y);
         const R cf = (R)a.coef;
+        if constexpr (P == P_F64) {
+          // chunk by chunk: the operand's 16 bytes live at a time, not 48 registers (in FP32 the
+          // 24 loads in flight together are worth more: hop_xpay 74 us, 82 us chunk by chunk)
+          constexpr int RPC = T::RPC;
 #pragma unroll
-        for (int c = 0; c < 24; ++c) {
-          const R g = (EPI == E_XPAY_G5 && c >= 12) ? -cf : cf;
-          y[c] += g * acc[c];
-          part += y[c] * y[c];
+          for (int k = 0; k < T::NCH; ++k) {
+            R y[RPC];
+            load_chunk<P>(F(a.y), cb, s, Ns, k, y);
+#pragma unroll
+            for (int j = 0; j < RPC; ++j) {
+              y[j] += (EPI == E_XPAY_G5 && k * RPC + j >= 12 ? -cf : cf) * acc[k * RPC + j];
+              part += y[j] * y[j];
+            }
+            store_chunk<P>(F(a.out), cb, s, Ns, k, y);
+          }
+        } else {
+          R y[24];
+          load_sp<P>(F(a.y), cb, s, Ns, y);
+#pragma unroll
+          for (int c = 0; c < 24; ++c) {
+            const R g = (EPI == E_XPAY_G5 && c >= 12) ? -cf : cf;
+            y[c] += g * acc[c];
+            part += y[c] * y[c];
+          }
+          store_sp<P>(F(a.out), cb, s, Ns, y);
         }
-        store_sp<P>(F(a.out), cb, s, Ns, y);
       } else if constexpr (EPI == E_M_XPAY) {
-        R y[24];
-        load_sp<P>(F(a.y), cb, s, Ns, y);
+        if constexpr (!T::HALF) {
+          constexpr int RPC = T::RPC;
 #pragma unroll
-        for (int c = 0; c < 24; ++c) y[c] += acc[c];
-        store_sp<P>(F(a.out), cb, s, Ns, y);
+          for (int k = 0; k < T::NCH; ++k) {
+            R y[RPC];
+            load_chunk<P>(F(a.y), cb, s, Ns, k, y);
+#pragma unroll
+            for (int j = 0; j < RPC; ++j) y[j] += acc[k * RPC + j];
+            store_chunk<P>(F(a.out), cb, s, Ns, k, y);
+          }
+        } else {
+          R y[24];
+          load_sp<P>(F(a.y), cb, s, Ns, y);
+#pragma unroll
+          for (int c = 0; c < 24; ++c) y[c] += acc[c];
+          store_sp<P>(F(a.out), cb, s, Ns, y);
+        }
       } else if constexpr (EPI == E_CG_UPDATE) {
         // alpha = (r, r) / (p, A p) was formed once by the reduction that produced (p, A p)
         R alpha;
