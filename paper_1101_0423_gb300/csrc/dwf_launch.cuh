@@ -97,10 +97,11 @@ cudaError_t hop_go(const HopArgs &a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// the inner-CG kernels get a compile-time Ns for the fifth-dimension extents in use
+// the inner CG's kernels and those of C get a compile-time Ns for the fifth-dimension extents in
+// use (C's second hop at 16^3x32x16: 126 registers and 124 us with Ns at run time)
 template <int P, int EPI>
 cudaError_t hop_ns(const HopArgs &a, cudaStream_t st) {
-  if constexpr (P != P_F64 && (EPI == E_M || EPI == E_XPAY_G5 || EPI == E_CG_UPDATE)) {
+  if constexpr (P != P_F64 && (EPI == E_M || EPI == E_XPAY_G5 || EPI == E_CG_UPDATE || EPI == E_M_XPAY)) {
     switch (a.Ns) {
       case 8: return hop_go<P, EPI, 8>(a, st);
       case 12: return hop_go<P, EPI, 12>(a, st);
