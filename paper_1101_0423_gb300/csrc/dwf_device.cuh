@@ -85,6 +85,21 @@ struct CGScalars {
 // reasons for an FP64 restart
 enum { RS_NONE = 0, RS_DELTA = 1, RS_TARGET = 2, RS_CAP = 3, RS_DIVERGED = 4, RS_STALLED = 5 };
 
+// ------------------------------------------------------------------ overlapped launches
+//
+// The kernels of an operator or a CG iteration are launched with programmatic stream
+// serialization: a kernel whose predecessor's CTAs have all called pdl_trigger() or ended may
+// start, set up what no kernel of the chain writes (the matrix along s, the tile's links and
+// neighbour indices) and then waits in pdl_wait() until its predecessors have completed and
+// their writes are visible.  The trigger stands at the end of a kernel's main work: there the
+// set-up hides behind the last CTAs and the reduction's tail (FP32 CG iteration at 8^4x16: 40.8
+// -> 36.2 us, at 16^3x32x16 429 -> 423 us).  At the start of the kernels it let later kernels'
+// CTAs pile up on whatever SM had room (51.7 and 468 us).  Nothing a predecessor writes is read, and nothing at all is written, before
+// pdl_wait(); field loads are plain (ld.global.nc promises data that is constant for the whole
+// launch, which such a launch cannot).  Without the launch attribute both are no-ops.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ------------------------------------------------------------------ spinor access
 
 template <int P>
@@ -106,39 +121,6 @@ __device__ __forceinline__ void load_sp(const Field f, long cb, int s, int Ns,
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       uint4 c = b[(size_t)k * Ns];
-      uint32_t w[4] = {c.x, c.y, c.z, c.w};
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float2 v;
-        if constexpr (P == P_F16) v = __half22float2(*reinterpret_cast<__half2 *>(&w[j]));
-        else v = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162 *>(&w[j]));
-        o[8 * k + 2 * j] = v.x * nm;
-        o[8 * k + 2 * j + 1] = v.y * nm;
-      }
-    }
-  }
-}
-
-// read-only variant for kernel inputs that no thread writes during the launch
-template <int P>
-__device__ __forceinline__ void load_sp_ro(const Field f, long cb, int s, int Ns,
-                                           typename PT<P>::real (&o)[24]) {
-  using T = PT<P>;
-  const typename T::chunk *b = (const typename T::chunk *)f.v + (size_t)cb * T::NCH * Ns + s;
-  if constexpr (P == P_F64) {
-#pragma unroll
-    for (int k = 0; k < 12; ++k) { double2 c = __ldg(b + (size_t)k * Ns); o[2 * k] = c.x; o[2 * k + 1] = c.y; }
-  } else if constexpr (P == P_F32) {
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      float4 c = __ldg(b + (size_t)k * Ns);
-      o[4 * k] = c.x; o[4 * k + 1] = c.y; o[4 * k + 2] = c.z; o[4 * k + 3] = c.w;
-    }
-  } else {
-    const float nm = __ldg(f.nrm + (size_t)cb * Ns + s);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      uint4 c = __ldg(b + (size_t)k * Ns);
       uint32_t w[4] = {c.x, c.y, c.z, c.w};
 #pragma unroll
       for (int j = 0; j < 4; ++j) {

@@ -559,6 +559,7 @@ dwf_status hop(dwf_ctx *c, cudaStream_t st, int prec, int epi, HopArgs a, int cl
     a.shape_threads = shape.threads;
     a.shape_persistent = shape.persistent ? 1 : 0;
   }
+  a.pdl = 1;
   Timed t(c, st, cls);
   CK(hop_any(prec, epi, a, st));
   return DWF_OK;
@@ -603,6 +604,7 @@ dwf_status smix(dwf_ctx *c, cudaStream_t st, int prec, int mode, Field in, Field
   set_smat(a, c, prec, kind, kind2);
   a.coef = coef;
   a.use_flag = use_flag;
+  a.pdl = 1;
   Timed t(c, st, cls);
   CK(smix_any(prec, mode, a, st));
   return DWF_OK;
@@ -1294,6 +1296,7 @@ dwf_status cg_iteration(dwf_ctx *c, cudaStream_t st, const SolveState &S, const 
     m.xfstride = field_bytes(c, xprec(P));
     set_smat(m, c, P, MK_M5T);
     m.use_flag = 1;
+    m.pdl = 1;
     m.sc = sl.d_sc;
     m.nrhs = S.K;
     m.fstride = fs;
@@ -2391,6 +2394,7 @@ extern "C" dwf_status dwf_apply_eo_dev_static(dwf_ctx *c, int op, int prec, int 
     a.sc = sc;
     a.partials = part;
     a.ticket = ticket;
+    a.pdl = 1;
     return hop_any(prec, epi, a, st);
   };
   auto smix_s = [&](int mode, Field x, Field o, int kind) -> cudaError_t {
@@ -2400,6 +2404,7 @@ extern "C" dwf_status dwf_apply_eo_dev_static(dwf_ctx *c, int op, int prec, int 
     a.out = o;
     set_smat(a, c, prec, kind);
     a.sc = sc;
+    a.pdl = 1;
     return smix_any(prec, mode, a, st);
   };
   // Eq. 11 on Schur parity sp: C v = v - M5 D M5 D v (u = -1/2 M5 H v, out = v + 1/2 M5 H u)

@@ -215,6 +215,7 @@ struct HopArgs {
   int Ns;
   int fin;             // FIN_* of the reduction
   int use_flag;        // honour CGScalars::restart_flag (skip work once set)
+  int pdl;             // launch may overlap its predecessor's end (pdl_wait)
   uint32_t wait_tries; // bound of each wait for a tile's copies, in mbarrier polls
   int skip_copies;     // failure-detection hook: issue no copies, so every wait runs out
   CGScalars *sc;
@@ -377,7 +378,7 @@ __device__ __noinline__ void hop_site_f64(const Field in, const int *nb, int s, 
   double ps[24], W[18];
 #pragma unroll
   for (int d = 0; d < 8; ++d) {
-    load_sp_ro<P>(in, nb[d], s, Ns, ps);
+    load_sp<P>(in, nb[d], s, Ns, ps);
     load_link<P>(links + d * PT<P>::LREALS, W);
     const double S = d < 4 ? -1.0 : 1.0;
     switch (d & 3) {
@@ -420,8 +421,6 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
   int sl, s;  // this thread's site of the tile and s-slice in the hop phase
   hop_thread<F2>(tid, Ns, spb, sl, s);
   const long ntile = (a.h + spb - 1) / spb;
-
-  if (a.use_flag && sc_->restart_flag) return;  // uniform over the grid
 
   constexpr bool PST = hop_persistent<EPI>();
   constexpr int NB = PST ? 2 : 1;  // link / neighbour buffers
@@ -498,10 +497,13 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
     }
   }
   __syncthreads();
-  if (tid == 0) {
-    if (!a.skip_copies) issue(blockIdx.x, 0);
-    prefetch_ops(blockIdx.x);
+  if (tid == 0 && !a.skip_copies) issue(blockIdx.x, 0);
+  pdl_wait();
+  if (a.use_flag && sc_->restart_flag) {  // uniform over the grid
+    if (tid == 0 && !a.skip_copies) mbar_wait(bar, 0, a.wait_tries);  // the copies in flight
+    return;
   }
+  if (tid == 0) prefetch_ops(blockIdx.x);
 
   // tiles blockIdx.x, blockIdx.x + gridDim.x, ... in this order, so that the CTA's share of
   // a reduction is summed in a fixed order (one tile per CTA unless persistent)
@@ -581,7 +583,7 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
         for (int dd = 0; dd < 8; ++dd) {
           const int d = (dd >> 1) + 4 * (dd & 1);
           float ps1[24];
-          load_sp_ro<P>(F(a.in), nb[d], s, Ns, ps1);
+          load_sp<P>(F(a.in), nb[d], s, Ns, ps1);
           f2 ps[12];
 #pragma unroll
           for (int q = 0; q < 12; ++q) ps[q] = pk2(ps1[2 * q], ps1[2 * q + 1]);
@@ -610,7 +612,7 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
 #pragma unroll
           for (int back = 0; back < 2; ++back) {
             R ps[24];
-            load_sp_ro<P>(F(a.in), nb[mu + 4 * back], s, Ns, ps);
+            load_sp<P>(F(a.in), nb[mu + 4 * back], s, Ns, ps);
             const int4 *W = myW + 9 * (mu + 4 * back);
             switch (mu) {
               case 0: ok &= hop_dir_fixed<0>(ai, ex, ps, W, back); break;
@@ -926,6 +928,7 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
       }
     }
   }
+  pdl_trigger();
   if constexpr (E::has_red) grid_sum<R>(part, a.partials + rb * a.part_stride, a.ticket + rb, a.fin, sc_);
 }
 
@@ -948,6 +951,7 @@ struct SmixArgs {
   long h;
   int Ns;
   int use_flag;
+  int pdl;                // as in HopArgs
   CGScalars *sc;
   int nrhs;               // batches of right-hand sides as in HopArgs
   size_t fstride, nstride;
@@ -979,7 +983,6 @@ __global__ void __launch_bounds__(256) k_smix(const SmixArgs a) {
   const int nthr = blockDim.x * blockDim.y;
   const long cb = (long)blockIdx.x * spb + sl;
   const bool active = cb < a.h;
-  if (a.use_flag && sc_->restart_flag) return;
   constexpr bool dual = MODE == S_DUAL;
   R *sK = reinterpret_cast<R *>(sm);
   R *sB = reinterpret_cast<R *>(sm + ((((size_t)(dual ? 4 : 2) * Ns * Ns * sizeof(R)) + 15) & ~size_t(15)));
@@ -991,6 +994,8 @@ __global__ void __launch_bounds__(256) k_smix(const SmixArgs a) {
       for (int i = tid; i < 2 * Ns * Ns; i += nthr) sK[2 * Ns * Ns + i] = (R)a.coef * K2[i];
     }
   }
+  pdl_wait();
+  if (a.use_flag && sc_->restart_flag) return;
   R v[24];
   if (active) {
     if constexpr (MODE == S_CGP) {
@@ -1020,7 +1025,7 @@ __global__ void __launch_bounds__(256) k_smix(const SmixArgs a) {
       for (int c = 0; c < 24; ++c) v[c] = r[c] + beta * v[c];
       store_sp<P>(F(a.p), cb, s, Ns, v);
     } else {
-      load_sp_ro<P>(F(a.in), cb, s, Ns, v);
+      load_sp<P>(F(a.in), cb, s, Ns, v);
     }
     if constexpr (MODE == S_CGP || MODE == S_G5) {
 #pragma unroll
@@ -1032,6 +1037,7 @@ __global__ void __launch_bounds__(256) k_smix(const SmixArgs a) {
   }
   __syncthreads();
   if (!active) return;
+  pdl_trigger();
   const R *site = sB + (size_t)sl * Ns * 24;
   for (int which = 0; which < (dual ? 2 : 1); ++which) {
     const R *K = sK + which * 2 * Ns * Ns;
@@ -1071,7 +1077,6 @@ __global__ void __launch_bounds__(256) k_srec(const SmixArgs a) {
   const int tid = s + sl * Ns, nthr = Ns * spb;
   const long cb0 = (long)blockIdx.x * spb, cb = cb0 + sl;
   const bool active = cb < a.h;
-  if (a.use_flag && sc_->restart_flag) return;
   double2 *sV = reinterpret_cast<double2 *>(sm);
   double *sT = reinterpret_cast<double *>(sV + (size_t)spb * 12 * cs);
   for (int i = tid; i < 2 * Ns * RC_N; i += nthr) {
@@ -1080,6 +1085,8 @@ __global__ void __launch_bounds__(256) k_srec(const SmixArgs a) {
   }
   const size_t base = (size_t)cb * 12 * Ns + s;  // chunk k at base + k Ns
   double2 *mine = sV + (size_t)sl * 12 * cs + s;
+  pdl_wait();
+  if (a.use_flag && sc_->restart_flag) return;
   if (active) {
     if constexpr (MODE == S_CGP) {
       // x += alpha p (the previous step), p = r + beta p (as k_smix)
@@ -1101,7 +1108,7 @@ __global__ void __launch_bounds__(256) k_srec(const SmixArgs a) {
       const double2 *gi = static_cast<const double2 *>(F(a.in).v) + base;
 #pragma unroll
       for (int k = 0; k < 12; ++k) {
-        const double2 v = __ldg(gi + k * Ns);
+        const double2 v = gi[k * Ns];
         mine[k * cs] = MODE == S_G5 && k >= 6 ? make_double2(-v.x, -v.y) : v;
       }
     }
@@ -1114,6 +1121,7 @@ __global__ void __launch_bounds__(256) k_srec(const SmixArgs a) {
     s_recurrence(sV + (size_t)col * cs + (bwd ? Ns - 1 : 0), bwd ? -1 : 1, sT + chi * Ns * RC_N, Ns, a.kappa, a.form);
   }
   __syncthreads();
+  pdl_trigger();
   if (active) {
     double2 *go = static_cast<double2 *>(F(a.out).v) + base;
 #pragma unroll
@@ -1146,7 +1154,7 @@ __global__ void __launch_bounds__(256) k_norm2(const VecArgs v) {
   double part = 0;
   for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < v.n; i += (long)gridDim.x * blockDim.x) {
     R x[24];
-    load_sp_ro<P>(v.a, i / v.Ns, (int)(i % v.Ns), v.Ns, x);
+    load_sp<P>(v.a, i / v.Ns, (int)(i % v.Ns), v.Ns, x);
     R pr = 0;
 #pragma unroll
     for (int c = 0; c < 24; ++c) pr += x[c] * x[c];
@@ -1162,7 +1170,7 @@ __global__ void __launch_bounds__(256) k_convert(const VecArgs v) {
     const long cb = i / v.Ns;
     const int s = (int)(i % v.Ns);
     typename PT<PA>::real x[24];
-    load_sp_ro<PA>(v.a, cb, s, v.Ns, x);
+    load_sp<PA>(v.a, cb, s, v.Ns, x);
     typename PT<PB>::real y[24];
 #pragma unroll
     for (int c = 0; c < 24; ++c) y[c] = (typename PT<PB>::real)x[c];
@@ -1276,6 +1284,7 @@ __global__ void __launch_bounds__(256) k_pack(const double *host, Field out, Geo
     rows[q * HOST_ROW + (i - 12 * q)] = __ldg(src + base[l].x + (i - l * Ns * 12));
   }
   __syncthreads();
+  pdl_trigger();
   if (sl >= nsite) return;
   typename PT<P>::real v[24];
 #pragma unroll
@@ -1295,13 +1304,15 @@ __global__ void __launch_bounds__(256) k_unpack(Field in, double *host, Geom g, 
   double2 *rows = reinterpret_cast<double2 *>(sm);
   longlong2 *base = reinterpret_cast<longlong2 *>(rows + (size_t)spb * Ns * HOST_ROW);
   const long cb0 = (long)blockIdx.x * spb;
+  const int nsite = host_tile(g, p, cb0, base, tid);
+  pdl_wait();
   if (cb0 + sl < g.h) {
     typename PT<P>::real v[24];
-    load_sp_ro<P>(in, cb0 + sl, s, Ns, v);
+    load_sp<P>(in, cb0 + sl, s, Ns, v);
 #pragma unroll
     for (int k = 0; k < 12; ++k) rows[tid * HOST_ROW + k] = make_double2((double)v[2 * k], (double)v[2 * k + 1]);
   }
-  const int nsite = host_tile(g, p, cb0, base, tid);
+  __syncthreads();
   double2 *dst = reinterpret_cast<double2 *>(host);
   const int per = Ns * 12;
 #pragma unroll 6
@@ -1352,6 +1363,7 @@ __global__ void k_gauge(const double *U, typename PT<P>::lreal *G, Geom g, int p
 __global__ void __launch_bounds__(256) k_sdual(const SmixArgs a) {
   const int Ns = a.Ns, s = threadIdx.x;
   const long cb = (long)blockIdx.x * blockDim.y + threadIdx.y;
+  pdl_wait();
   if (cb >= a.h) return;
   const double2 *gi = static_cast<const double2 *>(a.in.v) + (size_t)cb * 12 * Ns;
   double2 *g1 = static_cast<double2 *>(a.out.v) + (size_t)cb * 12 * Ns + s;
@@ -1366,10 +1378,10 @@ __global__ void __launch_bounds__(256) k_sdual(const SmixArgs a) {
     const bool b1 = o1 != 0.0, b2 = o2 != 0.0;
 #pragma unroll
     for (int k = 6 * chi; k < 6 * chi + 6; ++k) {
-      const double2 v = __ldg(gi + k * Ns + s);
+      const double2 v = gi[k * Ns + s];
       double2 u1 = make_double2(d1 * v.x, d1 * v.y), u2 = make_double2(d2 * v.x, d2 * v.y);
       if (b1 || b2) {
-        const double2 w = __ldg(gi + k * Ns + sn);
+        const double2 w = gi[k * Ns + sn];
         if (b1) u1 = make_double2(fma(o1, w.x, u1.x), fma(o1, w.y, u1.y));
         if (b2) u2 = make_double2(fma(o2, w.x, u2.x), fma(o2, w.y, u2.y));
       }
@@ -1384,8 +1396,8 @@ __global__ void __launch_bounds__(256) k_diff_norm2(const VecArgs v) {
   double part = 0;
   for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < v.n; i += (long)gridDim.x * blockDim.x) {
     double x[24], y[24];
-    load_sp_ro<P_F64>(v.a, i / v.Ns, (int)(i % v.Ns), v.Ns, x);
-    load_sp_ro<P_F64>(v.b, i / v.Ns, (int)(i % v.Ns), v.Ns, y);
+    load_sp<P_F64>(v.a, i / v.Ns, (int)(i % v.Ns), v.Ns, x);
+    load_sp<P_F64>(v.b, i / v.Ns, (int)(i % v.Ns), v.Ns, y);
     for (int c = 0; c < 24; ++c) part += (x[c] - y[c]) * (x[c] - y[c]);
   }
   grid_sum(part, v.partials, v.ticket, v.fin, v.sc);

@@ -38,6 +38,22 @@ inline int vec_grid(long n, int sm_count) {
   return (int)(g < 1 ? 1 : g);
 }
 
+// a launch, overlapping its predecessor's end if pdl (see pdl_wait)
+template <typename... A, typename... B>
+cudaError_t launch(void (*k)(A...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl, const B &...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, A(args)...);
+}
+
 template <int P, int EPI, int NSC>
 cudaError_t hop_go(const HopArgs &a, cudaStream_t st) {
   // the shape the host chose (autotuner), else 128-thread CTAs, persistent without M5
@@ -93,8 +109,7 @@ cudaError_t hop_go(const HopArgs &a, cudaStream_t st) {
     const long per_cta = (ntile + res - 1) / res;
     nblk = (ntile + per_cta - 1) / per_cta;
   }
-  k_hop<P, EPI, NSC><<<dim3((unsigned)nblk, nrhs), dim3(a.Ns, spb), smem, st>>>(a);
-  return cudaGetLastError();
+  return launch(k_hop<P, EPI, NSC>, dim3((unsigned)nblk, nrhs), dim3(a.Ns, spb), smem, st, a.pdl, a);
 }
 
 // the inner CG's kernels and those of C get a compile-time Ns for the fifth-dimension extents in
@@ -144,8 +159,7 @@ cudaError_t smix_go(const SmixArgs &a, cudaStream_t st) {
     }
   }
   const long nblk = (a.h + spb - 1) / spb;
-  k_smix<P, MODE><<<dim3((unsigned)nblk, a.nrhs > 1 ? a.nrhs : 1), dim3(a.Ns, spb), smem, st>>>(a);
-  return cudaGetLastError();
+  return launch(k_smix<P, MODE>, dim3((unsigned)nblk, a.nrhs > 1 ? a.nrhs : 1), dim3(a.Ns, spb), smem, st, a.pdl, a);
 }
 
 // FP64 recurrences: CTAs of about 128 threads, so that several share an SM and one's loads
@@ -165,8 +179,7 @@ cudaError_t srec_go(const SmixArgs &a, cudaStream_t st) {
     }
   }
   const long nblk = (a.h + spb - 1) / spb;
-  k_srec<MODE><<<dim3((unsigned)nblk, a.nrhs > 1 ? a.nrhs : 1), dim3(a.Ns, spb), smem, st>>>(a);
-  return cudaGetLastError();
+  return launch(k_srec<MODE>, dim3((unsigned)nblk, a.nrhs > 1 ? a.nrhs : 1), dim3(a.Ns, spb), smem, st, a.pdl, a);
 }
 
 cudaError_t sdual_launch(const SmixArgs &a, cudaStream_t st);
@@ -228,9 +241,8 @@ cudaError_t pack_launch(const double *host, Field out, Geom g, int parity, cudaS
 template <int P>
 cudaError_t unpack_launch(Field in, double *host, Geom g, int parity, int zero_other, cudaStream_t st) {
   const int spb = sites_per_block(P_F64, g.Ns);
-  k_unpack<P><<<(unsigned)((g.h + spb - 1) / spb), dim3(g.Ns, spb), host_stage_bytes(spb, g.Ns), st>>>(in, host, g, parity,
-                                                                                                    zero_other);
-  return cudaGetLastError();
+  return launch(k_unpack<P>, dim3((unsigned)((g.h + spb - 1) / spb)), dim3(g.Ns, spb), host_stage_bytes(spb, g.Ns), st, true,
+                in, host, g, parity, zero_other);
 }
 
 template <int P>

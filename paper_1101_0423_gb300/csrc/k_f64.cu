@@ -9,8 +9,7 @@ DWF_INSTANTIATE_PREC(P_F64)
 
 cudaError_t sdual_launch(const SmixArgs &a, cudaStream_t st) {
   const int spb = sites_per_block(P_F64, a.Ns);
-  k_sdual<<<(unsigned)((a.h + spb - 1) / spb), dim3(a.Ns, spb), 0, st>>>(a);
-  return cudaGetLastError();
+  return launch(k_sdual, dim3((unsigned)((a.h + spb - 1) / spb)), dim3(a.Ns, spb), 0, st, a.pdl, a);
 }
 
 cudaError_t neighbours_launch(int *nbr, Geom g, int parity, int sm_count, cudaStream_t st) {
