@@ -216,6 +216,7 @@ struct HopArgs {
   int fin;             // FIN_* of the reduction
   int use_flag;        // honour CGScalars::restart_flag (skip work once set)
   int pdl;             // launch may overlap its predecessor's end (pdl_wait)
+  int rev;             // walk the tiles from the last to the first
   uint32_t wait_tries; // bound of each wait for a tile's copies, in mbarrier polls
   int skip_copies;     // failure-detection hook: issue no copies, so every wait runs out
   CGScalars *sc;
@@ -434,8 +435,9 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
   // tile t's links and neighbour indices arrive in buffer b with two TMA bulk copies (both
   // contiguous and 16-byte sized); its epilogue operands are prefetched into L2 when the
   // tile starts
+  auto first_site = [&](long t) { return (a.rev ? ntile - 1 - t : t) * spb; };
   auto issue = [&](long t, int b) {
-    const long c0 = t * spb;
+    const long c0 = first_site(t);
     const int ns_t = (int)min((long)spb, a.h - c0);
     const uint32_t lbytes = (uint32_t)SM::raw(ns_t), nbytes = (uint32_t)ns_t * 8 * 4;
     mbar_expect_tx(bar + b, lbytes + nbytes);
@@ -443,7 +445,7 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
     bulk_g2s(sNb(b), a.nbr + c0 * 8, nbytes, bar + b);
   };
   auto prefetch_ops = [&](long t) {
-    const long c0 = t * spb;
+    const long c0 = first_site(t);
     const int ns_t = (int)min((long)spb, a.h - c0);
     const uint32_t ob = (uint32_t)((size_t)ns_t * T::NCH * Ns * 16);
     const size_t off = (size_t)c0 * T::NCH * Ns * 16;
@@ -512,7 +514,7 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
   for (long tile = blockIdx.x; tile < ntile; tile += gridDim.x, ++it) {
     const int bsel = PST ? (it & 1) : 0;
     const uint32_t par = PST ? (uint32_t)((it >> 1) & 1) : (uint32_t)(it & 1);
-    const long cb0 = tile * spb;
+    const long cb0 = first_site(tile);
     const int nsite = (int)min((long)spb, a.h - cb0);
     const bool active = sl < nsite;
     const long cb = cb0 + sl;
@@ -951,7 +953,7 @@ struct SmixArgs {
   long h;
   int Ns;
   int use_flag;
-  int pdl;                // as in HopArgs
+  int pdl, rev;           // as in HopArgs
   CGScalars *sc;
   int nrhs;               // batches of right-hand sides as in HopArgs
   size_t fstride, nstride;
@@ -981,7 +983,7 @@ __global__ void __launch_bounds__(256) k_smix(const SmixArgs a) {
   const int s = threadIdx.x, sl = threadIdx.y, spb = blockDim.y;
   const int tid = threadIdx.x + threadIdx.y * blockDim.x;
   const int nthr = blockDim.x * blockDim.y;
-  const long cb = (long)blockIdx.x * spb + sl;
+  const long cb = (long)(a.rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * spb + sl;
   const bool active = cb < a.h;
   constexpr bool dual = MODE == S_DUAL;
   R *sK = reinterpret_cast<R *>(sm);
