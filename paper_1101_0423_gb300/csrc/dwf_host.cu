@@ -539,6 +539,7 @@ HopArgs hop_args(dwf_ctx *c, int prec, int outpar) {
   a.Ns = c->Ns;
   a.fin = FIN_RED2;
   a.sc = c->d_sc;
+  a.host_err = c->h_err;
   a.partials = c->d_part;
   a.ticket = c->d_ticket;
   a.wait_tries = c->wait_tries;
@@ -683,6 +684,7 @@ dwf_status op_cdag(dwf_ctx *c, cudaStream_t st, int prec, int sp, Field v, Field
   b.y = v;
   b.out = q;
   b.coef = 0.5;
+  b.fin = FIN_NONE;
   TRY(hop(c, st, prec, E_XPAY_G5, b, cls));
   return DWF_OK;
 }
@@ -867,6 +869,8 @@ dwf_status dwf_create(const int dims[4], int Ns, double m0, double mq, const dou
   if ((e = dmalloc((void **)&c->d_sc, sizeof(CGScalars), c->device, c->stream)) != cudaSuccess) return bail(e);
   if (!(c->h_sc = static_cast<CGScalars *>(pinned_get(sizeof(CGScalars))))) return bail(cudaErrorMemoryAllocation);
   memset(c->h_sc, 0, sizeof(CGScalars));
+  if (!(c->h_err = static_cast<int *>(pinned_get(2 * sizeof(int))))) return bail(cudaErrorMemoryAllocation);
+  c->h_err[0] = c->h_err[1] = 0;
   c->part_len = std::max<size_t>((size_t)c->h, 8192);
   if ((e = dmalloc((void **)&c->d_part, c->part_len * sizeof(double), c->device, c->stream)) != cudaSuccess)
     return bail(e);
@@ -904,6 +908,7 @@ dwf_status dwf_destroy(dwf_ctx *c) {
     cudaStreamSynchronize(c->stream);
   }
   pinned_put(c->h_sc, sizeof(CGScalars));
+  pinned_put(c->h_err, 2 * sizeof(int));
   pinned_put(c->h_scb, c->h_scb_cap * sizeof(CGScalars));
   pinned_put(c->h_face, c->h_face_bytes);
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
@@ -1086,6 +1091,7 @@ dwf_status dwf_apply_eo_dev(dwf_ctx *c, int op, int prec, int parity, const doub
   TRY(ensure_gauge(c, prec, st));
   const Geom g = geom(c);
   const int cls = DWF_KC_OTHER;
+  c->h_err[0] = 0;
 
   Field in[2], out[2], tA, tB, tC;
   for (int p = 0; p < 2; ++p) {
@@ -1150,8 +1156,9 @@ dwf_status dwf_apply_eo_dev(dwf_ctx *c, int op, int prec, int parity, const doub
       TRY(unpack(1));
       break;
   }
+  // one wait; the kernels' error word is in host memory already
   CK(cudaStreamSynchronize(st));
-  return pull_scalars(c, st);
+  return c->h_err[0] ? pull_scalars(c, st) : DWF_OK;
 }
 
 dwf_status dwf_apply_eo(dwf_ctx *c, int op, int prec, int parity, const double *in, double *out) {
@@ -1369,14 +1376,14 @@ dwf_status tune_inner(dwf_ctx *c, cudaStream_t st, const SolveState &S) {
   x.y = S.p;
   x.out = S.q;
   x.coef = 0.5;
-  x.fin = FIN_NONE;
+  x.fin = FIN_RED2;
   HopArgs u = hop_args(c, P, S.sp);
   u.in = S.u;
   u.y = S.q;
   u.r = S.r;
   set_m5(u, c, P, false);
   u.coef = 0.5;
-  u.fin = FIN_NONE;
+  u.fin = FIN_RED2;
   const std::pair<int, HopArgs *> classes[3] = {{E_M, &m}, {E_XPAY_G5, &x}, {E_CG_UPDATE, &u}};
   cudaEvent_t e0 = next_event(c), e1 = next_event(c);
   for (const auto &cl : classes) {
@@ -2383,10 +2390,9 @@ extern "C" dwf_status dwf_apply_eo_dev_static(dwf_ctx *c, int op, int prec, int 
   unsigned *ticket = reinterpret_cast<unsigned *>(cur);
 
   cudaStream_t st = stream ? (cudaStream_t)stream : c->stream;
-  // the array keeps the previous call's contents: the scalars (error word included) and the
-  // ticket must start at zero
-  CK(cudaMemsetAsync(sc, 0, sizeof(CGScalars), st));
-  CK(cudaMemsetAsync(ticket, 0, sizeof(unsigned), st));
+  // the array keeps the previous call's contents: nothing here reads the scalars, no launch
+  // takes a reduction (so the ticket is not used), and errors come through host memory
+  c->h_err[1] = 0;
   const Geom g = geom(c);
   Field &in = f[0], &out = f[1], &tA = f[2], &tB = f[3], &tC = f[4];
   const int inpar = op == DWF_OP_DEO ? 1 : op == DWF_OP_DOE ? 0 : parity;
@@ -2402,6 +2408,8 @@ extern "C" dwf_status dwf_apply_eo_dev_static(dwf_ctx *c, int op, int prec, int 
     a.sc = sc;
     a.partials = part;
     a.ticket = ticket;
+    a.host_err = c->h_err + 1;
+    a.fin = FIN_NONE;
     a.pdl = 1;
     return hop_any(prec, epi, a, st);
   };
@@ -2450,12 +2458,10 @@ extern "C" dwf_status dwf_apply_eo_dev_static(dwf_ctx *c, int op, int prec, int 
       break;
   }
   CK(unpack_any(prec, out, d_out, g, outpar, true, st));
-  // the call returns when its work is done: it waits for `stream` and reads the kernels'
-  // error word (a bounded device-side wait that gave up) into host memory of its own
-  int err = 0;
-  CK(cudaMemcpyAsync(&err, &sc->error, sizeof(int), cudaMemcpyDeviceToHost, st));
+  // the call returns when its work is done: it waits for `stream`, after which the kernels'
+  // error word (a bounded device-side wait that gave up) is in host memory
   CK(cudaStreamSynchronize(st));
-  if (err) return fail(c, DWF_ETIMEOUT, "a device-side wait for the TMA link copy timed out");
+  if (c->h_err[1]) return fail(c, DWF_ETIMEOUT, "a device-side wait for the TMA link copy timed out");
   return DWF_OK;
 }
 

@@ -82,6 +82,7 @@ struct dwf_ctx {
   std::map<std::string, dwf::Buf> bufs;
   dwf::CGScalars *d_sc = nullptr;
   dwf::CGScalars *h_sc = nullptr;  // pinned mirror
+  int *h_err = nullptr;            // pinned error words: of operator calls, and of the static ones
   dwf::CGScalars *h_scb = nullptr; // pinned mirror of the scalars of a batch
   int h_scb_cap = 0;
   double *d_part = nullptr;

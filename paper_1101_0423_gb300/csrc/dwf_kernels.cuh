@@ -213,13 +213,14 @@ struct HopArgs {
   double coef;         // scale of H (plain/xpay) or of the matrix (M5 epilogues)
   long h;              // sites per parity
   int Ns;
-  int fin;             // FIN_* of the reduction
+  int fin;             // FIN_* of the reduction (FIN_NONE: none is taken)
   int use_flag;        // honour CGScalars::restart_flag (skip work once set)
   int pdl;             // launch may overlap its predecessor's end (pdl_wait)
   int rev;             // walk the tiles from the last to the first
   uint32_t wait_tries; // bound of each wait for a tile's copies, in mbarrier polls
   int skip_copies;     // failure-detection hook: issue no copies, so every wait runs out
   CGScalars *sc;
+  int *host_err;       // error word in pinned host memory (may be null), beside CGScalars::error
   double *partials;
   unsigned *ticket;
   // batches of right-hand sides: blockIdx.y selects one; its fields start fstride bytes
@@ -534,7 +535,10 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
     {
       const bool ok = mbar_wait(bar + bsel, par, a.wait_tries);
       if (__syncthreads_or(!ok)) {
-        if (tid == 0) atomicExch(&sc_->error, ERR_TMA_TIMEOUT);
+        if (tid == 0) {
+          atomicExch(&sc_->error, ERR_TMA_TIMEOUT);
+          if (a.host_err) *static_cast<volatile int *>(a.host_err) = ERR_TMA_TIMEOUT;
+        }
         mbar_wait(bar + bsel, par, a.wait_tries);  // the copy in flight
         return;
       }
@@ -931,7 +935,8 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
     }
   }
   pdl_trigger();
-  if constexpr (E::has_red) grid_sum<R>(part, a.partials + rb * a.part_stride, a.ticket + rb, a.fin, sc_);
+  if constexpr (E::has_red)
+    if (a.fin != FIN_NONE) grid_sum<R>(part, a.partials + rb * a.part_stride, a.ticket + rb, a.fin, sc_);
 }
 
 // ------------------------------------------------------------------ s-mixing kernel
