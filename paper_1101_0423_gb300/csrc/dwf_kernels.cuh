@@ -1016,7 +1016,10 @@ __global__ void __launch_bounds__(256) k_smix(const SmixArgs a) {
         beta = sc_->beta_f;
         alpha = sc_->alpha_f;
       }
+      // (r is loaded before x is stored: a load does not move ahead of a store that might alias)
       load_sp<P>(F(a.p), cb, s, Ns, v);
+      R r[24];
+      load_sp<P>(F(a.r), cb, s, Ns, r);
       {
         constexpr int PX = x_prec<P>();
         const Field fx = rb ? field_rhs(a.x, rb, a.xfstride, 0) : a.x;
@@ -1026,8 +1029,6 @@ __global__ void __launch_bounds__(256) k_smix(const SmixArgs a) {
         for (int c = 0; c < 24; ++c) xx[c] += alpha * v[c];
         store_sp<PX>(fx, cb, s, Ns, xx);
       }
-      R r[24];
-      load_sp<P>(F(a.r), cb, s, Ns, r);
 #pragma unroll
       for (int c = 0; c < 24; ++c) v[c] = r[c] + beta * v[c];
       store_sp<P>(F(a.p), cb, s, Ns, v);
@@ -1383,17 +1384,19 @@ __global__ void __launch_bounds__(256) k_sdual(const SmixArgs a) {
     const double kc = j ? a.coef : a.coef * a.kappa;
     const double d1 = a.coef * T1[RC_A], o1 = kc * T1[RC_B], d2 = a.coef * T2[RC_A], o2 = kc * T2[RC_B];
     const bool b1 = o1 != 0.0, b2 = o2 != 0.0;
+    double2 v[6], w[6];  // all loads before the first store, which might alias them
 #pragma unroll
-    for (int k = 6 * chi; k < 6 * chi + 6; ++k) {
-      const double2 v = gi[k * Ns + s];
-      double2 u1 = make_double2(d1 * v.x, d1 * v.y), u2 = make_double2(d2 * v.x, d2 * v.y);
-      if (b1 || b2) {
-        const double2 w = gi[k * Ns + sn];
-        if (b1) u1 = make_double2(fma(o1, w.x, u1.x), fma(o1, w.y, u1.y));
-        if (b2) u2 = make_double2(fma(o2, w.x, u2.x), fma(o2, w.y, u2.y));
-      }
-      g1[k * Ns] = u1;
-      g2[k * Ns] = u2;
+    for (int k = 0; k < 6; ++k) v[k] = gi[(6 * chi + k) * Ns + s];
+    if (b1 || b2)
+#pragma unroll
+      for (int k = 0; k < 6; ++k) w[k] = gi[(6 * chi + k) * Ns + sn];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      double2 u1 = make_double2(d1 * v[k].x, d1 * v[k].y), u2 = make_double2(d2 * v[k].x, d2 * v[k].y);
+      if (b1) u1 = make_double2(fma(o1, w[k].x, u1.x), fma(o1, w[k].y, u1.y));
+      if (b2) u2 = make_double2(fma(o2, w[k].x, u2.x), fma(o2, w[k].y, u2.y));
+      g1[(6 * chi + k) * Ns] = u1;
+      g2[(6 * chi + k) * Ns] = u2;
     }
   }
 }
