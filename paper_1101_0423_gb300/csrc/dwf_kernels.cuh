@@ -723,7 +723,16 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
               const long cb2 = cb0 + sl2;
               R alpha = 0;
               if constexpr (EPI == E_CG_UPDATE) alpha = sc_->alpha_f;
+              // (operands of the three chunks are loaded before the first is stored: a load does not
+              // move ahead of a store that might alias it)
               auto emit = [&](int sv, const f2 (&o)[6]) {
+                R y[3][4], z[3][4];
+#pragma unroll
+                for (int kk = 0; kk < 3; ++kk) {
+                  if constexpr (EPI != E_M) load_chunk<P>(F(a.y), cb2, sv, Ns, 3 * chi + kk, y[kk]);
+                  if constexpr (EPI == E_CG_UPDATE) load_chunk<P>(F(a.r), cb2, sv, Ns, 3 * chi + kk, z[kk]);
+                  if constexpr (EPI == E_RESID) load_chunk<P>(F(a.b), cb2, sv, Ns, 3 * chi + kk, z[kk]);
+                }
 #pragma unroll
                 for (int kk = 0; kk < 3; ++kk) {
                   const int k = 3 * chi + kk;
@@ -733,32 +742,19 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
                   if constexpr (EPI == E_M) {
                     store_chunk<P>(F(a.out), cb2, sv, Ns, k, v);
                   } else if constexpr (EPI == E_M_XPAY) {
-                    R y[4];
-                    load_chunk<P>(F(a.y), cb2, sv, Ns, k, y);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) v[j] += y[j];
+                    for (int j = 0; j < 4; ++j) v[j] += y[kk][j];
                     store_chunk<P>(F(a.out), cb2, sv, Ns, k, v);
-                  } else if constexpr (EPI == E_CG_UPDATE) {
-                    // Ap = y + K H; r -= alpha Ap (alpha formed with (p, A p))
-                    R y[4], r[4];
-                    load_chunk<P>(F(a.y), cb2, sv, Ns, k, y);
-                    load_chunk<P>(F(a.r), cb2, sv, Ns, k, r);
+                  } else {
+                    // CG update: Ap = y + K H; r -= alpha Ap (alpha formed with (p, A p)); residual:
+                    // b - (y + K H)
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                      r[j] -= alpha * (y[j] + v[j]);
-                      part += r[j] * r[j];
+                      if constexpr (EPI == E_CG_UPDATE) z[kk][j] -= alpha * (y[kk][j] + v[j]);
+                      else z[kk][j] -= y[kk][j] + v[j];
+                      part += z[kk][j] * z[kk][j];
                     }
-                    store_chunk<P>(F(a.r), cb2, sv, Ns, k, r);
-                  } else if constexpr (EPI == E_RESID) {
-                    R y[4], bb[4];
-                    load_chunk<P>(F(a.y), cb2, sv, Ns, k, y);
-                    load_chunk<P>(F(a.b), cb2, sv, Ns, k, bb);
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                      bb[j] -= y[j] + v[j];
-                      part += bb[j] * bb[j];
-                    }
-                    store_chunk<P>(F(a.out), cb2, sv, Ns, k, bb);
+                    store_chunk<P>(EPI == E_CG_UPDATE ? F(a.r) : F(a.out), cb2, sv, Ns, k, z[kk]);
                   }
                 }
               };
@@ -843,84 +839,72 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
         store_sp<P>(F(a.out), cb, s, Ns, acc);
       } else if constexpr (EPI == E_M) {
         store_sp<P>(F(a.out), cb, s, Ns, acc);
+      } else if constexpr (!T::HALF && !(P == P_F32 && !E::has_m)) {
+        // some 16-byte chunks at a time: their operands are loaded together, before the first is
+        // stored (a load does not move ahead of a store that might alias it), without holding
+        // a register for every real of them.  FP32 without M5 has room for all 24 below
+        // (hop_xpay 74 us, 82 us chunk by chunk).
+        constexpr int RPC = T::RPC, B = P == P_F64 ? 4 : 3;
+        constexpr bool two = EPI == E_CG_UPDATE || EPI == E_RESID;
+        const R cf = (R)a.coef;
+        R alpha = 0;
+        if constexpr (EPI == E_CG_UPDATE) {
+          // alpha = (r, r) / (p, A p) was formed once by the reduction that produced (p, A p)
+          // (x += alpha p is deferred to the next iteration's p-update, which reads p anyway)
+          if constexpr (P == P_F64) alpha = sc_->alpha;
+          else alpha = sc_->alpha_f;
+        }
+#pragma unroll
+        for (int k0 = 0; k0 < T::NCH; k0 += B) {
+          R y[B][RPC], z[B][RPC];
+#pragma unroll
+          for (int k = 0; k < B; ++k) {
+            load_chunk<P>(F(a.y), cb, s, Ns, k0 + k, y[k]);
+            if constexpr (two) load_chunk<P>(EPI == E_CG_UPDATE ? F(a.r) : F(a.b), cb, s, Ns, k0 + k, z[k]);
+          }
+#pragma unroll
+          for (int k = 0; k < B; ++k) {
+#pragma unroll
+            for (int j = 0; j < RPC; ++j) {
+              const int c = (k0 + k) * RPC + j;
+              R &o = two ? z[k][j] : y[k][j];
+              if constexpr (EPI == E_XPAY_G5 || EPI == E_XPAY) o += (EPI == E_XPAY_G5 && c >= 12 ? -cf : cf) * acc[c];
+              else if constexpr (EPI == E_M_XPAY) o += acc[c];
+              else if constexpr (EPI == E_CG_UPDATE) o -= alpha * (y[k][j] + acc[c]);
+              else o -= y[k][j] + acc[c];
+              part += o * o;
+            }
+            store_chunk<P>(EPI == E_CG_UPDATE ? F(a.r) : F(a.out), cb, s, Ns, k0 + k, two ? z[k] : y[k]);
+          }
+        }
       } else if constexpr (EPI == E_XPAY_G5 || EPI == E_XPAY) {
         const R cf = (R)a.coef;
-        if constexpr (P == P_F64) {
-          // chunk by chunk: the operand's 16 bytes live at a time, not 48 registers (in FP32 the
-          // 24 loads in flight together are worth more: hop_xpay 74 us, 82 us chunk by chunk)
-          constexpr int RPC = T::RPC;
+        R y[24];
+        load_sp<P>(F(a.y), cb, s, Ns, y);
 #pragma unroll
-          for (int k = 0; k < T::NCH; ++k) {
-            R y[RPC];
-            load_chunk<P>(F(a.y), cb, s, Ns, k, y);
-#pragma unroll
-            for (int j = 0; j < RPC; ++j) {
-              y[j] += (EPI == E_XPAY_G5 && k * RPC + j >= 12 ? -cf : cf) * acc[k * RPC + j];
-              part += y[j] * y[j];
-            }
-            store_chunk<P>(F(a.out), cb, s, Ns, k, y);
-          }
-        } else {
-          R y[24];
-          load_sp<P>(F(a.y), cb, s, Ns, y);
-#pragma unroll
-          for (int c = 0; c < 24; ++c) {
-            const R g = (EPI == E_XPAY_G5 && c >= 12) ? -cf : cf;
-            y[c] += g * acc[c];
-            part += y[c] * y[c];
-          }
-          store_sp<P>(F(a.out), cb, s, Ns, y);
+        for (int c = 0; c < 24; ++c) {
+          const R g = (EPI == E_XPAY_G5 && c >= 12) ? -cf : cf;
+          y[c] += g * acc[c];
+          part += y[c] * y[c];
         }
+        store_sp<P>(F(a.out), cb, s, Ns, y);
       } else if constexpr (EPI == E_M_XPAY) {
-        if constexpr (!T::HALF) {
-          constexpr int RPC = T::RPC;
+        R y[24];
+        load_sp<P>(F(a.y), cb, s, Ns, y);
 #pragma unroll
-          for (int k = 0; k < T::NCH; ++k) {
-            R y[RPC];
-            load_chunk<P>(F(a.y), cb, s, Ns, k, y);
-#pragma unroll
-            for (int j = 0; j < RPC; ++j) y[j] += acc[k * RPC + j];
-            store_chunk<P>(F(a.out), cb, s, Ns, k, y);
-          }
-        } else {
-          R y[24];
-          load_sp<P>(F(a.y), cb, s, Ns, y);
-#pragma unroll
-          for (int c = 0; c < 24; ++c) y[c] += acc[c];
-          store_sp<P>(F(a.out), cb, s, Ns, y);
-        }
+        for (int c = 0; c < 24; ++c) y[c] += acc[c];
+        store_sp<P>(F(a.out), cb, s, Ns, y);
       } else if constexpr (EPI == E_CG_UPDATE) {
-        // alpha = (r, r) / (p, A p) was formed once by the reduction that produced (p, A p)
-        R alpha;
-        if constexpr (P == P_F64) alpha = sc_->alpha;
-        else alpha = sc_->alpha_f;
-        // (x += alpha p is deferred to the next iteration's p-update, which reads p anyway)
-        if constexpr (!T::HALF) {
-          // chunk by chunk: two operands of 16 bytes live at a time, not 2 x 24 reals
-          constexpr int RPC = T::RPC;
+        const R alpha = sc_->alpha_f;
+        R y[24], r[24];
+        load_sp<P>(F(a.y), cb, s, Ns, y);
+        load_sp<P>(F(a.r), cb, s, Ns, r);
 #pragma unroll
-          for (int k = 0; k < T::NCH; ++k) {
-            R y[RPC], r[RPC];
-            load_chunk<P>(F(a.y), cb, s, Ns, k, y);
-            load_chunk<P>(F(a.r), cb, s, Ns, k, r);
-#pragma unroll
-            for (int j = 0; j < RPC; ++j) {
-              r[j] -= alpha * (y[j] + acc[k * RPC + j]);
-              part += r[j] * r[j];
-            }
-            store_chunk<P>(F(a.r), cb, s, Ns, k, r);
-          }
-        } else {
-          R y[24], r[24];
-          load_sp<P>(F(a.y), cb, s, Ns, y);
-          load_sp<P>(F(a.r), cb, s, Ns, r);
-#pragma unroll
-          for (int c = 0; c < 24; ++c) {
-            r[c] -= alpha * (y[c] + acc[c]);
-            part += r[c] * r[c];
-          }
-          store_sp<P>(F(a.r), cb, s, Ns, r);
+        for (int c = 0; c < 24; ++c) {
+          r[c] -= alpha * (y[c] + acc[c]);
+          part += r[c] * r[c];
         }
+        store_sp<P>(F(a.r), cb, s, Ns, r);
       } else if constexpr (EPI == E_RESID) {
         R y[24], bb[24];
         load_sp<P>(F(a.y), cb, s, Ns, y);
