@@ -325,11 +325,13 @@ __device__ __forceinline__ void hop_thread(int tid, int Ns, int spb, int &sl, in
 }
 // kernels without an M5 epilogue run persistent CTAs (measured: hop_xpay 96 -> 79 us); the
 // M5 kernels keep one tile per CTA and the smaller footprint (a double-buffered persistent
-// form took hop_m5 93 -> 104 us and hop_update 158 -> 188 us by shrinking the L1)
-template <int EPI> constexpr bool hop_persistent() { return !EpiT<EPI>::has_m; }
+// form took hop_m5 93 -> 104 us and hop_update 158 -> 188 us by shrinking the L1), and so do the
+// FP64 kernels, whose tiles last long enough that the last wave of persistent CTAs is felt
+// (D in FP64 at 24^3x48x8: 4.91 -> 4.42 ms)
+template <int P, int EPI> constexpr bool hop_persistent() { return !EpiT<EPI>::has_m && P != P_F64; }
 template <int P, int EPI>
 __host__ __device__ inline size_t hop_smem_bytes(int spb, int Ns) {
-  return HopSmem<P>::bytes(spb, Ns, hop_persistent<EPI>() ? 2 : 1, EpiT<EPI>::has_m);
+  return HopSmem<P>::bytes(spb, Ns, hop_persistent<P, EPI>() ? 2 : 1, EpiT<EPI>::has_m);
 }
 
 // the recurrence of RC_A along one column of two reals, in place: col[0], col[step], ... are
@@ -424,7 +426,7 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
   hop_thread<F2>(tid, Ns, spb, sl, s);
   const long ntile = (a.h + spb - 1) / spb;
 
-  constexpr bool PST = hop_persistent<EPI>();
+  constexpr bool PST = hop_persistent<P, EPI>();
   constexpr int NB = PST ? 2 : 1;  // link / neighbour buffers
   uint64_t *bar = reinterpret_cast<uint64_t *>(sm);  // bar[b]: buffer b's copies landed
   float4 *sP = reinterpret_cast<float4 *>(sm + SM::off_exp(spb, NB));

@@ -55,9 +55,9 @@ cudaError_t launch(void (*k)(A...), dim3 grid, dim3 block, size_t smem, cudaStre
 
 template <int P, int EPI, int NSC>
 cudaError_t hop_go(const HopArgs &a, cudaStream_t st) {
-  // the shape the host chose (autotuner), else 128-thread CTAs, persistent without M5
+  // the shape the host chose (autotuner), else 128-thread CTAs, persistent without M5 (not FP64)
   int spb = hop_sites_per_block(P, a.Ns);
-  bool persistent = hop_persistent<EPI>();
+  bool persistent = hop_persistent<P, EPI>();
   if (a.shape_threads > 0) {
     spb = std::max(1, std::min(64, a.shape_threads / a.Ns));
     persistent = a.shape_persistent != 0;
