@@ -6,7 +6,8 @@
 //            with fused epilogues: M5 (Sec. 3.3), vector add/sub (Sec. 3.5), CG update and
 //            the block partial sums of the reductions (Sec. 3.4).
 //   k_smix   per-site matrices along s (M5, M5^T, S1, S2, omega + sigma L, ...), with the
-//            CG direction update p = r + beta p fused in front.
+//            CG direction update p = r + beta p fused in front; in FP64 k_srec (recurrence
+//            along s) and k_sdual (two bidiagonal matrices) instead.
 //   k_pack / k_unpack  host layout <-> device layout (Sec. 3.1), precision conversion.
 //   k_norm2, k_accum, k_convert  reductions and vector updates.
 // Reductions: per-thread partials promoted to FP64, warp shuffles, block sums written to
@@ -253,10 +254,10 @@ __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~size_t(
 // (links and indices arrive by TMA bulk copies).  FP32 kernels use the links as copied (padded
 // to 80 bytes, so the nine complex entries are five aligned float4); the 16-bit forms rebuild
 // each link's third row and expand the tile's links into that same FP32 form; FP64 kernels
-// convert them to fixed point once for the Ns threads of a site.  The M5 staging rows overlay everything from offset 64 on (kernels
-// with an M5 epilogue take one tile per CTA, so the link buffers are dead by then).  Shared
-// memory is kept small on purpose: what the CTAs leave of the SM's 256 KB is the L1 that
-// holds the neighbour gathers in flight.
+// convert them to fixed point once for the Ns threads of a site.  The M5 staging rows overlay
+// everything from offset 64 on (kernels with an M5 epilogue take one tile per CTA, so the link
+// buffers are dead by then).  Shared memory is kept small on purpose: what the CTAs leave of the
+// SM's 256 KB is the L1 that holds the neighbour gathers in flight.
 template <int P> struct HopSmem {
   static constexpr bool F2 = !(P == P_F64);
   using RL = typename PT<P>::real;
