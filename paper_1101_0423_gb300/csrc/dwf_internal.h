@@ -11,12 +11,10 @@
 #include "../../include/dwf.h"
 #include "dwf_launch.cuh"
 #include "dwf_part.cuh"
+#include "dwf_smat.h"
 #include "dwf_tune.h"
 
 namespace dwf {
-
-// matrices along s held per context (kernel order K[chi][t][s] on the device)
-enum MatKind { MK_M5 = 0, MK_M5T, MK_S1, MK_S2, MK_W, MK_Z, MK_ID, MK_MASS, MK_COUNT };
 
 struct Buf {
   void *v = nullptr;
@@ -59,20 +57,12 @@ struct dwf_gauge {
   int refs = 1;  // the creator's reference plus one per attached context
 };
 
-struct dwf_ctx {
+struct dwf_ctx : dwf::SMatrices {
   int dims[4];
-  int Ns;
   long V4, h;
-  double m0, mq;
-  std::vector<double> omega, sigma;
-  // host FP64 matrices, row-major [chi][s][t]
-  std::vector<double> mat[dwf::MK_COUNT];
   // device matrices per arithmetic precision (0: double, 1: float), kernel order
   void *dmat[2][dwf::MK_COUNT] = {};
-  // the same as FP64 recurrence tables along s (RC_A); empty where there is none
-  std::vector<double> rec[dwf::MK_COUNT];
-  double *drec[dwf::MK_COUNT] = {};
-  bool rec_tight[dwf::MK_COUNT] = {};  // as accurate as the dense matrix: used by s-mixing too
+  double *drec[dwf::MK_COUNT] = {};  // recurrence tables (FP64); null where there is none
   int *d_nbr[2] = {nullptr, nullptr};
   double *d_U = nullptr;  // FP64 host-layout copy of the gauge field
   void *d_gauge[4][2] = {};

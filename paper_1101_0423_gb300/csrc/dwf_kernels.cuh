@@ -16,6 +16,7 @@
 #pragma once
 
 #include "dwf_device.cuh"
+#include "dwf_smat.h"
 
 namespace dwf {
 
@@ -192,13 +193,6 @@ template <int EPI> struct EpiT {
   static constexpr bool has_red = EPI == E_XPAY_G5 || EPI == E_CG_UPDATE || EPI == E_RESID;
 };
 
-// FP64 recurrence along s (one table per matrix: per chirality Ns steps, step j at s = j, or
-// Ns - 1 - j for a chirality that runs backward), two or three FP64 operations a real and step
-// and one for the closure, against Ns for the dense row:
-//   z_j = A_j v_j + B_j v_{j-1} - C_j z_{j-1},  u_j = z_j + R_j z_{j-1},
-// where step 0 takes v_{-1} = kappa v_{Ns-1} and z_{-1} = kappa z_{Ns-1}, with z_{Ns-1} known
-// beforehand from the closure z_{Ns-1} = sum_j W_j v_j
-enum { RC_A, RC_B, RC_C, RC_R, RC_W, RC_N = 6 };
 // which coefficients a table has: B = 0 (M5, S1, S2) or R = 0 (M5^T)
 enum { REC_SOLVE_MUL = 0, REC_MUL_SOLVE = 1 };
 

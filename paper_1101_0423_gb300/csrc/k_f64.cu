@@ -8,6 +8,7 @@ namespace dwf {
 DWF_INSTANTIATE_PREC(P_F64)
 
 cudaError_t sdual_launch(const SmixArgs &a, cudaStream_t st) {
+  if (!a.rec || !a.rec2) return cudaErrorInvalidValue;
   const int spb = sites_per_block(a.Ns);
   return launch(k_sdual, dim3((unsigned)((a.h + spb - 1) / spb)), dim3(a.Ns, spb), 0, st, a.pdl, a);
 }

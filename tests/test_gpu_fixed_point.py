@@ -120,3 +120,18 @@ def test_matrices_along_s(gpu_lib, opname, ns, ratio):
     else:
         want = oracle.apply_s(dims, ns, mp, mm, x, transpose=opname == "M5T", parity=1)
     assert np.abs(got - want).max() <= 1e-14 * max(1.0, np.abs(want).max())
+
+
+def test_whole_operator_where_the_dense_corner_cancels(gpu_lib):
+    """D(mq) in FP64 for a mass and weights at which (d - m0) sigma is 1 to three digits and the
+    corner |kappa| = 500: the bidiagonal matrices come from their tables (the dense Z agrees with
+    its own to 5e-14 only).  Each output is a sum of products whose largest, |kappa| |psi| and
+    sigma |kappa| |H psi|, cancel to 1e-3 of themselves at worst: within 100 of their roundings."""
+    dwf, dims, ns, m0, mq = gpu_lib, (2, 4, 2, 6), 8, 1e-3, 1.0
+    om, sg = np.ones(ns), np.ones(ns) / 3.999
+    U = inputs.gauge_field(dims, 0.5, seed=62)
+    x = inputs.gaussian_source(dims, ns, seed=63)
+    with dwf.Context(dims, ns, m0, mq, om, sg, U) as ctx:
+        got = dwf.dwf_apply_eo(ctx.h, dwf.OP_DFULL, dwf.PREC_F64, 1, x)
+    want = oracle.dfull(dims, ns, U, m0, mq, om, sg, x)
+    assert np.abs(got - want).max() <= 100 * 1.2e-16 * 500 * np.abs(x).max()
