@@ -40,6 +40,10 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
       "l"(src), "r"(bytes), "r"(smem_u32(bar))
       : "memory");
 }
+// orders this thread's own accesses to shared memory before bulk copies into the same bytes that
+// are issued after the next barrier (the copies write through the async proxy, which a barrier
+// alone does not order after ordinary stores)
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 // bounded wait on phase `ph`; false if the bound ran out
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t ph, uint32_t max_tries) {
   for (uint32_t i = 0; i < max_tries; ++i) {
@@ -249,8 +253,9 @@ __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~size_t(
 // to 80 bytes, so the nine complex entries are five aligned float4); the 16-bit forms rebuild
 // each link's third row and expand the tile's links into that same FP32 form; FP64 kernels
 // convert them to fixed point once for the Ns threads of a site.  The M5 staging rows overlay
-// everything from offset 64 on (kernels with an M5 epilogue take one tile per CTA, so the link
-// buffers are dead by then).  Shared memory is kept small on purpose: what the CTAs leave of the
+// everything from offset 64 on (kernels with an M5 epilogue have one buffer, which is dead by
+// then; a CTA that walks several tiles refills it after the barrier and the proxy fence at the
+// top of the tile loop).  Shared memory is kept small on purpose: what the CTAs leave of the
 // SM's 256 KB is the L1 that holds the neighbour gathers in flight.
 template <int P> struct HopSmem {
   static constexpr bool F2 = !(P == P_F64);
@@ -391,9 +396,10 @@ __device__ __noinline__ void hop_site_f64(const Field in, const int *nb, int s, 
   for (int c = 0; c < 24; ++c) out[c] = acc[c];
 }
 
-// k_hop: one thread per (site, s), CTA = (Ns, spb) = one tile of spb sites (kernels without
-// an M5 epilogue: a grid of as many CTAs as fit on the GPU at once, walking all tiles).  Per
-// tile: eight gathers of the neighbours' spinors (Eq. 12), the hop sum in packed FP32 pairs or
+// k_hop: one thread per (site, s), CTA = (Ns, spb) = one tile of spb sites at a time: one tile
+// per CTA, or a persistent grid of as many CTAs as fit on the GPU at once, walking all tiles
+// (the default of the FP32 and 16-bit kernels without an M5 epilogue; the autotuner may choose
+// either for every kernel of the inner CG).  Per tile: eight gathers of the neighbours' spinors (Eq. 12), the hop sum in packed FP32 pairs or
 // FP64 fixed point, the epilogue.  The FP64
 // forms (fixed-point products, FP64 projections and M5) are capped at 128 registers, four CTAs
 // per SM: a CTA's M5 phase keeps the FP64 pipe busy while others are in their integer hop
@@ -520,6 +526,7 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
     const int *sN = sNb(bsel);
     if constexpr (!PST) {
       if (it > 0) {  // one buffer: the previous tile must be finished before it is refilled
+        fence_proxy_async();
         __syncthreads();
         if (tid == 0) {
           if (!a.skip_copies) issue(tile, 0);

@@ -48,3 +48,31 @@ def test_untuned_query_reports_the_default(gpu_lib):
         with pytest.raises(dwf.DwfError) as e:
             dwf.dwf_tuned_shape(ctx.h, dwf.PREC_F64, dwf.KC_HOP_M5)
         assert e.value.status == dwf.DWF_EINVAL
+
+
+@pytest.mark.parametrize("ns", [2, 8])
+def test_operators_keep_their_results_under_tuned_shapes(gpu_lib, ns):
+    """Operators take the shapes that a solve tuned: on a lattice of several tiles per resident
+    CTA (a CTA then refills its link buffer over the rows it staged) C and C^dag stay bit for bit
+    what the allocation-free entry point, which keeps the default shapes, gives (Ns = 2; Ns = 8
+    is over that one's size, and is compared with FP64)."""
+    import torch
+    dwf, dims = gpu_lib, (16, 16, 16, 32)
+    om, sg = inputs.weights("shamir", ns)
+    x = torch.from_numpy(inputs.gaussian_source(dims, ns, seed=81)).cuda()
+    with dwf.Context(dims, ns, M0, 0.1, om, sg, inputs.gauge_field(dims, 0.3, seed=80)) as ctx:
+        sol = torch.empty_like(x)
+        dwf.dwf_solve_dev(ctx.h, x, sol, tol=1e-6)
+        assert dwf.dwf_tuned_shape(ctx.h, dwf.PREC_F32, dwf.KC_HOP_M5)[2]
+        for op in (dwf.OP_C, dwf.OP_CDAG):
+            want, got = torch.empty_like(x), torch.empty_like(x)
+            if ns == 2:
+                dwf.dwf_apply_eo_dev_static(ctx.h, op, dwf.PREC_F32, 1, x, want)
+            else:
+                dwf.dwf_apply_eo_dev(ctx.h, op, dwf.PREC_F64, 1, x, want)
+            for _ in range(20):
+                dwf.dwf_apply_eo_dev(ctx.h, op, dwf.PREC_F32, 1, x, got)
+                if ns == 2:
+                    assert torch.equal(got, want)
+                else:
+                    assert float((got - want).abs().max()) <= 1e-5 * float(want.abs().max())
