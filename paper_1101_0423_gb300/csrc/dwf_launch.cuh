@@ -9,6 +9,7 @@
 #include <tuple>
 
 #include "dwf_kernels.cuh"
+#include "dwf_optin.h"
 
 namespace dwf {
 
@@ -53,6 +54,18 @@ cudaError_t launch(void (*k)(A...), dim3 grid, dim3 block, size_t smem, cudaStre
   return cudaLaunchKernelEx(&cfg, k, A(args)...);
 }
 
+// allows kernel k `smem` bytes of dynamic shared memory on the current device
+template <typename... A>
+cudaError_t allow_smem(SmemOptIn &seen, void (*k)(A...), size_t smem) {
+  if (smem <= kSmemNoOptIn) return cudaSuccess;
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  return (cudaError_t)seen.ensure(dev, smem, [&] {
+    return (int)cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  });
+}
+
 template <int P, int EPI, int NSC>
 cudaError_t hop_go(const HopArgs &a, cudaStream_t st) {
   // the shape the host chose (autotuner), else 128-thread CTAs, persistent without M5 (not FP64)
@@ -64,17 +77,9 @@ cudaError_t hop_go(const HopArgs &a, cudaStream_t st) {
   }
   if (spb * a.Ns > 256) return cudaErrorInvalidConfiguration;
   const size_t smem = hop_smem_bytes<P, EPI>(spb, a.Ns);
-  if (smem > 48 * 1024) {  // launches may come from several host threads
-    static std::mutex cmu;
-    static size_t configured = 0;
-    std::lock_guard<std::mutex> lock(cmu);
-    if (configured < smem) {
-      cudaError_t e =
-          cudaFuncSetAttribute(k_hop<P, EPI, NSC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-      configured = smem;
-    }
-  }
+  static SmemOptIn optin;
+  cudaError_t e = allow_smem(optin, k_hop<P, EPI, NSC>, smem);
+  if (e != cudaSuccess) return e;
   const int nrhs = a.nrhs > 1 ? a.nrhs : 1;
   const long ntile = (a.h + spb - 1) / spb;
   long nblk = ntile;  // one tile per CTA
@@ -84,7 +89,7 @@ cudaError_t hop_go(const HopArgs &a, cudaStream_t st) {
     // a finished right-hand side's row returns at once)
     const int nthr = a.Ns * spb;
     int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     // resident CTAs per GPU for this kernel, CTA size and shared memory (cached)
     static std::mutex mu;
@@ -149,36 +154,19 @@ cudaError_t smix_go(const SmixArgs &a, cudaStream_t st) {
   // (4^4x8: 31.2 -> 29.4 us an iteration, 12 rows of 8^4x8: 77.1 -> 75.2 ms a solve)
   const int spb = sites_per_block(a.Ns);
   const size_t smem = smix_smem_bytes<P>(spb, a.Ns, MODE == S_DUAL);
-  if (smem > 48 * 1024) {
-    static std::mutex cmu;
-    static size_t configured = 0;
-    std::lock_guard<std::mutex> lock(cmu);
-    if (configured < smem) {
-      cudaError_t e = cudaFuncSetAttribute(k_smix<P, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-      configured = smem;
-    }
-  }
+  static SmemOptIn optin;
+  const cudaError_t e = allow_smem(optin, k_smix<P, MODE>, smem);
+  if (e != cudaSuccess) return e;
   const long nblk = (a.h + spb - 1) / spb;
   return launch(k_smix<P, MODE>, dim3((unsigned)nblk, a.nrhs > 1 ? a.nrhs : 1), dim3(a.Ns, spb), smem, st, a.pdl, a);
 }
 
 // FP64 recurrences: CTAs of about 128 threads, so that several share an SM and one's loads
-// overlap another's FP64 phase
+// overlap another's FP64 phase (at most 37 KB of shared memory, at Ns = 2)
 template <int MODE>
 cudaError_t srec_go(const SmixArgs &a, cudaStream_t st) {
   const int spb = sites_per_block(a.Ns);
   const size_t smem = srec_smem_bytes(spb, a.Ns);
-  if (smem > 48 * 1024) {
-    static std::mutex cmu;
-    static size_t configured = 0;
-    std::lock_guard<std::mutex> lock(cmu);
-    if (configured < smem) {
-      cudaError_t e = cudaFuncSetAttribute(k_srec<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-      configured = smem;
-    }
-  }
   const long nblk = (a.h + spb - 1) / spb;
   return launch(k_srec<MODE>, dim3((unsigned)nblk, a.nrhs > 1 ? a.nrhs : 1), dim3(a.Ns, spb), smem, st, a.pdl, a);
 }
