@@ -375,7 +375,6 @@ void set_m5(HopArgs &a, dwf_ctx *c, int prec, bool trans) {
   a.K = dmat(c, prec, trans ? MK_M5T : MK_M5);
   a.rec = c->drec[trans ? MK_M5T : MK_M5];
   a.mtrans = trans ? 1 : 0;
-  a.kappa = -c->mq / (2.0 * c->m0);
 }
 
 // the matrices along s of an s-mixing launch: dense, and as recurrence tables (FP64; a matrix
@@ -385,9 +384,7 @@ void set_smat(SmixArgs &a, dwf_ctx *c, int prec, int kind, int kind2 = MK_ID) {
   a.K2 = dmat(c, prec, kind2);
   a.rec = c->rec_tight[kind] ? c->drec[kind] : nullptr;
   a.rec2 = c->drec[kind2];
-  a.kappa = -c->mq / (2.0 * c->m0);
   a.mtrans = kind == MK_M5T ? 1 : 0;
-  a.form = kind == MK_M5T ? REC_MUL_SOLVE : REC_SOLVE_MUL;
   a.coef = 1.0;
   a.h = c->h;
   a.Ns = c->Ns;

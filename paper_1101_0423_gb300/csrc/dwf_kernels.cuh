@@ -197,9 +197,6 @@ template <int EPI> struct EpiT {
   static constexpr bool has_red = EPI == E_XPAY_G5 || EPI == E_CG_UPDATE || EPI == E_RESID;
 };
 
-// which coefficients a table has: B = 0 (M5, S1, S2) or R = 0 (M5^T)
-enum { REC_SOLVE_MUL = 0, REC_MUL_SOLVE = 1 };
-
 struct HopArgs {
   Field in, out, y, b, r;
   const void *gauge;   // doubled gauge of the output parity: [cb][SITE_LREALS], links [8][LREALS]
@@ -208,7 +205,6 @@ struct HopArgs {
   const void *rec;     // FP64: the same as a recurrence table along s, per chirality Ns
                        // steps of RC_N reals (see RC_A)
   int mtrans;          // 0: M5, 1: M5^T (direction of each chirality's recurrence)
-  double kappa;        // corner of L, -mq / (2 m0) (Eq. 4)
   double coef;         // scale of H (plain/xpay) or of the matrix (M5 epilogues)
   long h;              // sites per parity
   int Ns;
@@ -336,40 +332,23 @@ __host__ __device__ inline size_t hop_smem_bytes(int spb, int Ns) {
 
 // the recurrence of RC_A along one column of two reals, in place: col[0], col[step], ... are
 // its Ns values in the order of the steps
-__device__ __forceinline__ void s_recurrence(double2 *col, int step, const double *T, int Ns, double kappa, int form) {
-  double2 zp = make_double2(0.0, 0.0), vp = zp;
+__device__ __forceinline__ void s_recurrence(double2 *col, int step, const double *T, int Ns) {
+  double2 y = make_double2(0.0, 0.0);
 #pragma unroll 4
   for (int j = 0; j < Ns; ++j) {
-    vp = col[j * step];
+    const double2 v = col[j * step];
     const double w = T[j * RC_N + RC_W];
-    zp.x = fma(w, vp.x, zp.x);
-    zp.y = fma(w, vp.y, zp.y);
+    y.x = fma(w, v.x, y.x);
+    y.y = fma(w, v.y, y.y);
   }
-  zp.x *= kappa, zp.y *= kappa;
-  if (form == REC_SOLVE_MUL) {
 #pragma unroll 4
-    for (int j = 0; j < Ns; ++j) {
-      const double2 ab = *reinterpret_cast<const double2 *>(T + j * RC_N), cr = *reinterpret_cast<const double2 *>(T + j * RC_N + 2);
-      const double2 v = col[j * step];
-      double2 z, u;
-      z.x = fma(-cr.x, zp.x, ab.x * v.x);
-      z.y = fma(-cr.x, zp.y, ab.x * v.y);
-      u.x = fma(cr.y, zp.x, z.x);
-      u.y = fma(cr.y, zp.y, z.y);
-      zp = z;
-      col[j * step] = u;
-    }
-  } else {
-    vp.x *= kappa, vp.y *= kappa;
-#pragma unroll 4
-    for (int j = 0; j < Ns; ++j) {
-      const double2 ab = *reinterpret_cast<const double2 *>(T + j * RC_N), cr = *reinterpret_cast<const double2 *>(T + j * RC_N + 2);
-      const double2 v = col[j * step];
-      zp.x = fma(-cr.x, zp.x, fma(ab.y, vp.x, ab.x * v.x));
-      zp.y = fma(-cr.x, zp.y, fma(ab.y, vp.y, ab.x * v.y));
-      vp = v;
-      col[j * step] = zp;
-    }
+  for (int j = 0; j < Ns; ++j) {
+    const double2 ad = *reinterpret_cast<const double2 *>(T + j * RC_N);
+    const double e = T[j * RC_N + RC_E];
+    const double2 v = col[j * step];
+    col[j * step] = make_double2(fma(ad.x, v.x, y.x), fma(ad.x, v.y, y.y));
+    y.x = fma(-e, y.x, ad.y * v.x);
+    y.y = fma(-e, y.y, ad.y * v.y);
   }
 }
 
@@ -497,8 +476,7 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
       const R *Tg = static_cast<const R *>(a.rec);
       R *sT = reinterpret_cast<R *>(sKb);
       for (int i = tid; i < 2 * Ns * RC_N; i += nthr) {
-        const int e = i % RC_N;
-        sT[i] = (e == RC_A || e == RC_B || e == RC_W) ? a.coef * Tg[i] : Tg[i];
+        sT[i] = i % RC_N != RC_E ? a.coef * Tg[i] : Tg[i];
       }
     }
   }
@@ -824,8 +802,7 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
             const int chi = k >= NCK / 2 ? 1 : 0;
             const bool bwd = (chi ^ a.mtrans) != 0;
             double2 *col = reinterpret_cast<double2 *>(sB + (size_t)l * sstride + 2 * k) + (bwd ? (Ns - 1) * (ROW / 2) : 0);
-            s_recurrence(col, bwd ? -(ROW / 2) : ROW / 2, sT + chi * Ns * RC_N, Ns, a.kappa,
-                         a.mtrans ? REC_MUL_SOLVE : REC_SOLVE_MUL);
+            s_recurrence(col, bwd ? -(ROW / 2) : ROW / 2, sT + chi * Ns * RC_N, Ns);
           }
         }
         __syncthreads();
@@ -940,8 +917,7 @@ struct SmixArgs {
   Field in, out, out2, r, p, x;
   const void *K, *K2;  // K[chi][t][s]
   const double *rec, *rec2;  // FP64: the same as recurrence tables (RC_A); rec null: dense
-  double kappa;              // corner of L (Eq. 4)
-  int mtrans, form;          // rec is M5^T (direction of each chirality); REC_* form
+  int mtrans;                // rec is M5^T (direction of each chirality)
   double coef;
   long h;
   int Ns;
@@ -1076,8 +1052,7 @@ __global__ void __launch_bounds__(256) k_srec(const SmixArgs a) {
   double2 *sV = reinterpret_cast<double2 *>(sm);
   double *sT = reinterpret_cast<double *>(sV + (size_t)spb * 12 * cs);
   for (int i = tid; i < 2 * Ns * RC_N; i += nthr) {
-    const int e = i % RC_N;
-    sT[i] = (e == RC_A || e == RC_B || e == RC_W) ? a.coef * a.rec[i] : a.rec[i];
+    sT[i] = i % RC_N != RC_E ? a.coef * a.rec[i] : a.rec[i];
   }
   const size_t base = (size_t)cb * 12 * Ns + s;  // chunk k at base + k Ns
   double2 *mine = sV + (size_t)sl * 12 * cs + s;
@@ -1114,7 +1089,7 @@ __global__ void __launch_bounds__(256) k_srec(const SmixArgs a) {
   for (int col = tid; col < ncol; col += nthr) {
     const int chi = col % 12 >= 6 ? 1 : 0;
     const bool bwd = (chi ^ a.mtrans) != 0;
-    s_recurrence(sV + (size_t)col * cs + (bwd ? Ns - 1 : 0), bwd ? -1 : 1, sT + chi * Ns * RC_N, Ns, a.kappa, a.form);
+    s_recurrence(sV + (size_t)col * cs + (bwd ? Ns - 1 : 0), bwd ? -1 : 1, sT + chi * Ns * RC_N, Ns);
   }
   __syncthreads();
   pdl_trigger();
@@ -1127,7 +1102,7 @@ __global__ void __launch_bounds__(256) k_srec(const SmixArgs a) {
 
 // FP64 S_DUAL with two cyclic bidiagonal matrices (omega + sigma L and (d - m0)(omega + sigma L)
 // + 1 - L of Eq. 5, or 1 and d - m0): tables of RC_A with the diagonal in A and the factor of L
-// in B.  Two multiply-adds a real and matrix; each slice reads its neighbour along s through L1.
+// at the next step in D (W of the last step at the corner).  Two multiply-adds a real and matrix; each slice reads its neighbour along s through L1.
 __global__ void __launch_bounds__(256) k_sdual(const SmixArgs a);
 
 // ------------------------------------------------------------------ per-(site, s) vector kernels
@@ -1368,9 +1343,10 @@ __global__ void __launch_bounds__(256) k_sdual(const SmixArgs a) {
   for (int chi = 0; chi < 2; ++chi) {
     const int j = chi ? Ns - 1 - s : s;                                // step of this slice
     const int sn = chi ? (s + 1 < Ns ? s + 1 : 0) : (s ? s : Ns) - 1;  // (L v)_s reads v at sn
-    const double *T1 = a.rec + (chi * Ns + j) * RC_N, *T2 = a.rec2 + (chi * Ns + j) * RC_N;
-    const double kc = j ? a.coef : a.coef * a.kappa;
-    const double d1 = a.coef * T1[RC_A], o1 = kc * T1[RC_B], d2 = a.coef * T2[RC_A], o2 = kc * T2[RC_B];
+    const int at = (chi * Ns + j) * RC_N;
+    const int off = j ? at - RC_N + RC_D : (chi * Ns + Ns - 1) * RC_N + RC_W;
+    const double d1 = a.coef * a.rec[at + RC_A], o1 = a.coef * a.rec[off];
+    const double d2 = a.coef * a.rec2[at + RC_A], o2 = a.coef * a.rec2[off];
     const bool b1 = o1 != 0.0, b2 = o2 != 0.0;
     double2 v[6], w[6];  // all loads before the first store, which might alias them
 #pragma unroll

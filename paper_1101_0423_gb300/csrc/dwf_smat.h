@@ -16,12 +16,12 @@ constexpr double kD = 4.0;  // space-time dimension d of Eq. 2
 enum MatKind { MK_M5 = 0, MK_M5T, MK_S1, MK_S2, MK_W, MK_Z, MK_ID, MK_MASS, MK_COUNT };
 
 // FP64 recurrence along s (one table per matrix: per chirality Ns steps, step j at s = j, or
-// Ns - 1 - j for a chirality that runs backward), two or three FP64 operations a real and step
-// and one for the closure, against Ns for the dense row:
-//   z_j = A_j v_j + B_j v_{j-1} - C_j z_{j-1},  u_j = z_j + R_j z_{j-1},
-// where step 0 takes v_{-1} = kappa v_{Ns-1} and z_{-1} = kappa z_{Ns-1}, with z_{Ns-1} known
-// beforehand from the closure z_{Ns-1} = sum_j W_j v_j
-enum { RC_A, RC_B, RC_C, RC_R, RC_W, RC_N = 6 };
+// Ns - 1 - j for a chirality that runs backward), three FP64 operations a real and step and one
+// for the closure, against Ns for the dense row:
+//   u_j = A_j v_j + y_j,  y_{j+1} = D_j v_j - E_j y_j,  y_0 = sum_j W_j v_j (the closure, through
+// the corner kappa of L, Eq. 4).  The diagonal term enters u last, so u takes one rounding and
+// those of the smaller y
+enum { RC_A, RC_D, RC_E, RC_W, RC_N = 4 };
 
 struct SMatrices {
   int Ns = 0;
@@ -123,113 +123,168 @@ inline bool build_matrices(SMatrices *c) {
   return true;
 }
 
-// The fifth-dimension matrices as recurrences along s for the FP64 kernels (tables of RC_A).
-// With A = (d - m0) sqrt(omega) (1 + cL) + omega^{-1/2} (1 - L) (cyclic bidiagonal through the
-// corner kappa of L, Eq. 4; diagonal a, below it beta) and P = sqrt(omega) (1 + cL):
-// M5 = P A^{-1}, M5^T = A^{-T} P^T (Eq. 8), S1 = M5 omega^{-1/2}, S2 = (1 + cL)^{-1}
-// omega^{-1/2} (Eq. 9); and the bidiagonal matrices of Eq. 5.  A chirality's recurrence visits
-// s in one direction (step j at s = j, or Ns - 1 - j when backward: chirality - , or chirality
-// + for M5^T).  In P A^{-1} the solved z is kept as sqrt(omega) z, which leaves one
-// multiplication per step for P.
-inline void apply_recurrence(const double *T, int Ns, bool bwd, double kappa, const double *v, double *u) {
+// a number as the sum of two doubles, for the table entries: each then is within half a unit of
+// its last place, where products and quotients of rounded factors lose two or three units
+struct Dd {
+  double h, l;
+  Dd(double x = 0.0) : h(x), l(0.0) {}
+  Dd(double x, double y) : h(x + y), l(y - ((x + y) - x)) {}  // |x| >= |y|
+};
+inline Dd operator-(const Dd &a) {
+  Dd r;
+  r.h = -a.h, r.l = -a.l;
+  return r;
+}
+inline Dd operator+(const Dd &a, const Dd &b) {
+  const double s = a.h + b.h, t = s - a.h;
+  return Dd(s, ((a.h - (s - t)) + (b.h - t)) + (a.l + b.l));
+}
+inline Dd operator-(const Dd &a, const Dd &b) { return a + -b; }
+inline Dd operator*(const Dd &a, const Dd &b) {
+  const double p = a.h * b.h;
+  return Dd(p, std::fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h));
+}
+inline Dd operator/(const Dd &a, const Dd &b) {
+  const double q = a.h / b.h;
+  return Dd(q, (a - b * Dd(q)).h / b.h);
+}
+inline Dd sqrt_dd(double x) {
+  const double r = std::sqrt(x);
+  return Dd(r, std::fma(-r, r, x) / (2.0 * r));
+}
+
+// u = the recurrence of table T (one chirality) applied to v, operation for operation as the kernels
+inline void apply_recurrence(const double *T, int Ns, bool bwd, const double *v, double *u) {
   auto sg = [&](int j) { return bwd ? Ns - 1 - j : j; };
-  double zc = 0.0;
-  for (int j = 0; j < Ns; ++j) zc += T[j * RC_N + RC_W] * v[sg(j)];
-  double zp = kappa * zc, vp = kappa * v[sg(Ns - 1)];
+  double y = 0.0;
+  for (int j = 0; j < Ns; ++j) y = std::fma(T[j * RC_N + RC_W], v[sg(j)], y);
   for (int j = 0; j < Ns; ++j) {
     const double *t = T + j * RC_N;
-    const int s = sg(j);
-    const double z = t[RC_A] * v[s] + t[RC_B] * vp - t[RC_C] * zp;
-    u[s] = z + t[RC_R] * zp;
-    zp = z;
-    vp = v[s];
+    const double x = v[sg(j)];
+    u[sg(j)] = std::fma(t[RC_A], x, y);
+    y = std::fma(-t[RC_E], y, t[RC_D] * x);
   }
+}
+
+// one chirality's table.  With den = (d - m0) omega + 1, g = (sigma + omega) / (omega den) and
+// n, k the slices of the step before and after this one (at s):
+//   M5 = P A^{-1} (Eq. 8, P = sqrt(omega) (1 + cL)): A z = v in steps z = A_j v - C_j z', C =
+//     ((d - m0) sigma - 1) / den sqrt(omega / omega_n), then u = A_j v + G_j z' with G = g
+//     sqrt(omega / omega_n); y = G_j z' is kept, so that A = omega / den, D = G_{j+1} A_j, E =
+//     C_j G_{j+1} / G_j.  A step whose G is 0 or negligible (sigma = - omega) keeps 2^-60 of
+//     what it would be with |sigma| instead, which is below u's rounding.  S1 = M5 omega^{-1/2} scales A and D.
+//   M5^T = A^{-T} P^T: A as above, D = g sqrt(omega omega_k) / den_k, E = ((d - m0) sigma - 1) /
+//     den_k sqrt(omega_k / omega)
+//   S2 = (1 + cL)^{-1} omega^{-1/2} (Eq. 9): A = omega^{-1/2}, E = c_k = sigma_k / omega_k, D = - E A
+//   the bidiagonal matrices of Eq. 5: A the diagonal, D the factor of L at k, E = 0
+// false if the closure has no solution.
+inline bool recurrence_table(const SMatrices &c, int kind, int chi, double *T) {
+  const int Ns = c.Ns;
+  const bool bwd = (chi ^ (kind == MK_M5T)) != 0;
+  auto sg = [&](int j) { return bwd ? Ns - 1 - j : j; };
+  const Dd kappa = -(Dd(c.mq) / Dd(2.0 * c.m0)), dm = Dd(kD) - Dd(c.m0);
+  std::vector<Dd> A(Ns), D(Ns), E(Ns), G(Ns);
+  auto om = [&](int j) { return Dd(c.omega[sg(j)]); };
+  auto si = [&](int j) { return Dd(c.sigma[sg(j)]); };
+  auto rt = [&](int j) { return sqrt_dd(c.omega[sg(j)]); };
+  auto den = [&](int j) { return dm * om(j) + Dd(1.0); };
+  auto g = [&](int j) { return (si(j) + om(j)) / (om(j) * den(j)); };
+  for (int j = 0; j < Ns; ++j) {
+    const Dd x = rt(j) / rt((j + Ns - 1) % Ns);
+    const double least = std::ldexp((std::fabs(si(j).h) + om(j).h) / (om(j) * den(j) * x).h, -60);
+    G[j] = g(j) * x;
+    if (!(std::fabs(G[j].h) > least)) G[j] = Dd(least);
+  }
+  for (int j = 0; j < Ns; ++j) {
+    const int k = (j + 1) % Ns, n = (j + Ns - 1) % Ns;
+    switch (kind) {
+      case MK_M5:
+      case MK_S1:
+        A[j] = (kind == MK_M5 ? om(j) : rt(j)) / den(j);
+        D[j] = G[k] * A[j];
+        E[j] = (dm * si(j) - Dd(1.0)) / den(j) * (rt(j) / rt(n)) * (G[k] / G[j]);
+        break;
+      case MK_M5T:
+        A[j] = om(j) / den(j);
+        D[j] = g(j) * rt(j) * rt(k) / den(k);
+        E[j] = (dm * si(j) - Dd(1.0)) / den(k) * (rt(k) / rt(j));
+        break;
+      case MK_S2:
+        A[j] = Dd(1.0) / rt(j);
+        E[j] = si(k) / om(k);
+        D[j] = -(E[j] * A[j]);
+        break;
+      case MK_W: A[j] = om(j), D[j] = si(k); break;                                            // omega + sigma L
+      case MK_Z: A[j] = dm * om(j) + Dd(1.0), D[j] = dm * si(k) - Dd(1.0); break;  // (d - m0) of it + 1 - L
+      case MK_ID: A[j] = Dd(1.0); break;
+      case MK_MASS: A[j] = dm; break;
+    }
+  }
+  // closure: y_0 = kappa y_Ns, where y_Ns depends linearly on y_0 through every step
+  Dd q = kappa;
+  for (int j = 0; j < Ns; ++j) q = q * -E[j];
+  const Dd one_q = Dd(1.0) - q;
+  if (one_q.h == 0.0) return false;
+  Dd r = kappa / one_q;
+  for (int j = Ns - 1; j >= 0; --j) {
+    const Dd w = r * D[j];
+    r = r * -E[j];
+    if (Ns == 1) A[j] = A[j] + w;  // a single slice: one product
+    T[j * RC_N + RC_A] = A[j].h;
+    T[j * RC_N + RC_D] = Ns == 1 ? 0.0 : D[j].h;
+    T[j * RC_N + RC_E] = Ns == 1 ? 0.0 : E[j].h;
+    T[j * RC_N + RC_W] = Ns == 1 ? 0.0 : w.h;
+  }
+  return true;
 }
 
 // builds the tables and checks those with a solve against their dense matrices column by
 // column; S1 and S2 may have none, M5 and M5^T have to agree.  The bidiagonal matrices are
 // their tables' own entries, exact for every mass and weight, and always have one: the corner
 // of the dense Z, dm (sigma kappa) - kappa, cancels where dm sigma is near 1 and kappa large,
-// and says nothing about the table's (dm sigma - 1) kappa
+// and says nothing about the table's (dm sigma - 1) kappa.
+//
+// A table is tight, and the s-mixing kernel takes it, if it agrees with the dense matrix to the
+// latter's own few roundings and y_0's rounding, carried along s by the product of the E, stays
+// below the largest entry's.  Where sigma > omega that product grows along s and the dense rows
+// are the more accurate.  Tight tables err less than the rows (root mean square over random
+// fields, in units of 2^-52 of the result: Shamir 0.24 against 0.5-0.9 for Ns = 4 to 64, Borici
+// 0.27-0.29 against 0.4-0.9, cosine 0.29-0.36 against 0.9-1.2).
 inline bool build_recurrences(SMatrices *c) {
   const int Ns = c->Ns;
-  const double kappa = -c->mq / (2.0 * c->m0);
-  const double dm = kD - c->m0;
-  std::vector<double> a(Ns), beta(Ns), sw(Ns), cc(Ns), lam(Ns), u(Ns), v(Ns);
-  for (int s = 0; s < Ns; ++s) {
-    sw[s] = sqrt(c->omega[s]);
-    a[s] = dm * sw[s] + 1.0 / sw[s];
-    beta[s] = dm * c->sigma[s] / sw[s] - 1.0 / sw[s];
-    cc[s] = c->sigma[s] / c->omega[s];
-    if (a[s] == 0.0) return false;
-  }
+  std::vector<double> u(Ns), v(Ns);
   for (int kind = 0; kind < MK_COUNT; ++kind) {
     std::vector<double> &rec = c->rec[kind];
     rec.assign((size_t)2 * Ns * RC_N, 0.0);
+    bool ok = true, tight = true;
     double worst = 0.0;
-    bool ok = true;
     for (int chi = 0; chi < 2 && ok; ++chi) {
-      const bool bwd = (chi ^ (kind == MK_M5T)) != 0;
-      auto sg = [&](int j) { return bwd ? Ns - 1 - j : j; };
       double *T = rec.data() + (size_t)chi * Ns * RC_N;
-      for (int j = 0; j < Ns; ++j) {
-        const int s = sg(j), n = sg((j + Ns - 1) % Ns);  // this step's s and the step before's
-        double *t = T + j * RC_N;
-        if (kind == MK_M5T) {  // g = P^T v, then A^T z = g
-          t[RC_A] = sw[s] / a[s];
-          t[RC_B] = sw[n] * cc[n] / a[s];
-          t[RC_C] = beta[n] / a[s];
-        } else if (kind == MK_W || kind == MK_Z) {  // omega + sigma L; (d - m0) of it + 1 - L
-          t[RC_A] = kind == MK_W ? c->omega[s] : dm * c->omega[s] + 1.0;
-          t[RC_B] = kind == MK_W ? c->sigma[s] : dm * c->sigma[s] - 1.0;
-        } else if (kind == MK_ID || kind == MK_MASS) {
-          t[RC_A] = kind == MK_ID ? 1.0 : dm;
-        } else if (kind == MK_S2) {  // (1 + cL) z = omega^{-1/2} v
-          t[RC_A] = 1.0 / sw[s];
-          t[RC_C] = cc[s];
-        } else {  // A z = v (S1: omega^{-1/2} v), u = sqrt(omega) (z + c L z); sqrt(omega) z kept
-          t[RC_A] = (kind == MK_S1 ? 1.0 : sw[s]) / a[s];
-          t[RC_C] = beta[s] / a[s] * sw[s] / sw[n];
-          t[RC_R] = cc[s] * sw[s] / sw[n];
-        }
-      }
-      // closure: z_last depends linearly on z_{-1} = kappa z_last through every step
-      double q = -T[RC_C] * kappa;
-      for (int j = 1; j < Ns; ++j) q *= -T[j * RC_N + RC_C];
-      const double den = 1.0 - q;
-      ok = den != 0.0;
-      double r = 1.0;
-      for (int j = Ns - 1; j >= 0 && ok; --j) {
-        lam[j] = r / den;
-        r *= -T[j * RC_N + RC_C];
-      }
-      for (int j = 0; j < Ns && ok; ++j) {
-        double w = lam[j] * T[j * RC_N + RC_A];
-        if (j + 1 < Ns) w += lam[j + 1] * T[(j + 1) * RC_N + RC_B];
-        if (j == Ns - 1) w += kappa * lam[0] * T[RC_B];
-        T[j * RC_N + RC_W] = w;
-      }
-      // check: the recurrence reproduces every column of the dense matrix
+      ok = recurrence_table(*c, kind, chi, T);
+      if (!ok || kind >= MK_W) continue;
       const double *M = c->mat[kind].data() + (size_t)chi * Ns * Ns;
-      double mmax = 0.0;
+      double mmax = 0.0, wsum = 0.0, grow = 1.0, prod = 1.0;
       for (int i = 0; i < Ns * Ns; ++i) mmax = std::max(mmax, fabs(M[i]));
-      for (int t0 = 0; t0 < Ns && ok; ++t0) {
+      for (int j = 0; j < Ns; ++j) {
+        wsum += fabs(T[j * RC_N + RC_W]);
+        grow = std::max(grow, prod);
+        prod *= fabs(T[j * RC_N + RC_E]);
+      }
+      tight = tight && (grow <= 1.0 || wsum * grow <= mmax);
+      for (int t0 = 0; t0 < Ns; ++t0) {
         std::fill(v.begin(), v.end(), 0.0);
         v[t0] = 1.0;
-        apply_recurrence(T, Ns, bwd, kappa, v.data(), u.data());
+        apply_recurrence(T, Ns, (chi ^ (kind == MK_M5T)) != 0, v.data(), u.data());
         for (int s = 0; s < Ns; ++s)
           worst = std::max(worst, std::isfinite(u[s]) ? fabs(u[s] - M[s * Ns + t0]) / mmax : 1.0);
       }
     }
-    if (kind >= MK_W) worst = 0.0;
-    if (!ok || worst > 1e-11) {
+    // (a system is refused where the two differ by more: too ill conditioned for either)
+    if (!ok || worst > 2e-11) {
       if (kind == MK_M5 || kind == MK_M5T) return false;
       rec.clear();
     }
-    // where the recurrence grows along s (sigma > omega) it loses digits that the dense rows
-    // keep: the s-mixing kernel then takes those (Shamir, Borici and cosine weights up to
-    // Ns = 64 agree to 1e-15)
-    c->rec_tight[kind] = ok && worst <= 1e-14;
+    c->rec_tight[kind] = ok && tight && worst <= 1e-15;
   }
   return true;
 }

@@ -7,6 +7,8 @@ FP64 arithmetic in any order keeps it within 8 * 12 roundings of 2^-53 times the
 neighbour (times the link's norm), and the fixed-point form's truncation is below that: 1e-14
 of the largest neighbouring |psi| (about 90 * 1.1e-16), times the largest link row norm.
 """
+from fractions import Fraction
+
 import numpy as np
 import pytest
 
@@ -97,29 +99,72 @@ def test_values_that_are_not_finite(gpu_lib):
     assert (np.abs(got - want) <= bound)[~bad].all()
 
 
-@pytest.mark.parametrize("opname", ["M5", "M5T", "DFULL"])
-@pytest.mark.parametrize("ns,ratio", [(1, 1.0), (2, 0.0), (7, 1.0), (16, 1.0), (33, 0.5), (64, 1.0), (16, 1.8), (32, 1.8)])
+def exact_m5(ns, m0, mq, ratio):
+    """M5 of Eq. 8 per chirality for omega = 1, sigma = ratio, column by column in rationals: u = (1 +
+    cL) z with (a + b L) z = v, a = (d - m0) + 1, b = (d - m0) sigma - 1, and kappa = L's corner."""
+    F = Fraction
+    kappa, dm, sg = -F(mq) / (2 * F(m0)), 4 - F(m0), F(ratio)
+    a, b = dm + 1, dm * sg - 1
+    M = np.empty((ns, ns), dtype=object)
+    for t in range(ns):
+        f, g, fs, gs = F(0), F(1), [], []
+        for j in range(ns):
+            f, g = (F(int(j == t)) - b * f) / a, -b * g / a
+            fs.append(f), gs.append(g)
+        zl = fs[-1] / (1 - gs[-1] * kappa)
+        z = [x + y * kappa * zl for x, y in zip(fs, gs)]
+        for j in range(ns):
+            M[j, t] = z[j] + sg * (z[j - 1] if j else kappa * z[-1])
+    M = M.astype(float)
+    return M, M[::-1, ::-1].copy()  # chirality -: L^T, which runs the other way
+
+
+def rows_error(ns, m0, mq, ratio):
+    """Bound of the relative error of M5's rows and tables for omega = 1: a rounding made in the
+    solve along s comes round through the corner |kappa| grown by ((d - m0) sigma - 1) / ((d - m0)
+    + 1) a step where that is above 1, with Ns of them (45 roundings of the products besides)."""
+    grow = max(1.0, ((4 - m0) * ratio - 1) / (5 - m0)) ** ns
+    return 45 * 2.3e-16 + ns * 2.3e-16 * (grow - 1) * max(mq / (2 * m0), 1e-3)
+
+
+@pytest.mark.parametrize("opname", ["M5", "M5T", "C", "CDAG", "CCDAG", "DFULL"])
+@pytest.mark.parametrize("ns,ratio", [(1, 1.0), (2, 0.0), (7, 1.0), (16, 1.0), (33, 0.5), (64, 1.0), (16, 1.8),
+                                      (16, -1.0), (16, 3.0), (32, 2.4)])
 def test_matrices_along_s(gpu_lib, opname, ns, ratio):
-    """The FP64 s-mixing kernel as a recurrence and, where sigma > omega makes the recurrence
-    grow along s, dense: each output is a sum of Ns products, so 1e-14 (about 45 * 2 eps) of the
-    field's size times the matrix's.  The reference matrix is M5 = P A^{-1} with the cyclic
-    bidiagonal A = (d - m0) P + omega^{-1/2} (1 - L), P = sqrt(omega) (1 + cL): A's condition
-    number is below 60 for these weights, that of 1 + cL (which Eq. 8 inverts) up to 1.8^32."""
-    dwf, dims, mq = gpu_lib, (2, 4, 2, 6), 0.05
+    """The FP64 matrices along s as recurrences and, where sigma > omega lets the closure's
+    rounding grow along s (3.0 at Ns = 16, 2.4 at 32: test_smat_host.py), as dense rows in the
+    s-mixing kernel; the hop epilogues keep the recurrence.  M5 against exact rationals, each
+    M5 within rows_error of the field's and the matrix's size, each hop a factor of at most 8."""
+    dwf, dims, m0, mq = gpu_lib, (2, 4, 2, 6), 1.8, 0.05
     om, sg = np.ones(ns), ratio * np.ones(ns)
     U = inputs.gauge_field(dims, 0.5, seed=60)
     x = inputs.gaussian_source(dims, ns, seed=61)
-    L = np.diag(np.ones(ns - 1), -1)
-    L[0, -1] += -mq / (2 * 1.8)
-    P = [np.diag(np.sqrt(om)) @ (np.eye(ns) + np.diag(sg / om) @ l) for l in (L, L.T)]
-    mp, mm = [p @ np.linalg.inv(2.2 * p + np.diag(1 / np.sqrt(om)) @ (np.eye(ns) - l)) for p, l in zip(P, (L, L.T))]
-    with dwf.Context(dims, ns, 1.8, mq, om, sg, U) as ctx:
+    mp, mm = exact_m5(ns, m0, mq, ratio)
+    with dwf.Context(dims, ns, m0, mq, om, sg, U) as ctx:
         got = dwf.dwf_apply_eo(ctx.h, getattr(dwf, "OP_" + opname), dwf.PREC_F64, 1, x)
+    tol = rows_error(ns, m0, mq, ratio)
     if opname == "DFULL":
-        want = oracle.dfull(dims, ns, U, 1.8, mq, om, sg, x)
-    else:
+        want, tol = oracle.dfull(dims, ns, U, m0, mq, om, sg, x), 45 * 2.3e-16
+    elif opname in ("M5", "M5T"):
         want = oracle.apply_s(dims, ns, mp, mm, x, transpose=opname == "M5T", parity=1)
-    assert np.abs(got - want).max() <= 1e-14 * max(1.0, np.abs(want).max())
+    else:
+        # |out| of one hop and M5 pair is within 4 |M5| of its input: errors of both add up
+        want = {"C": oracle.c_op, "CDAG": oracle.cdag_op, "CCDAG": oracle.ccdag_op}[opname](dims, ns, U, mp, mm, 1, x)
+        m5 = max(1.0, np.abs(mp).sum(1).max())
+        tol *= 4 * (4 * m5) ** (4 if opname == "CCDAG" else 2) * np.abs(x).max() / np.abs(want).max()
+    assert np.abs(got - want).max() <= tol * max(1.0, np.abs(want).max())
+
+
+def test_solve_where_the_matrices_along_s_are_dense(gpu_lib):
+    """A full solve whose reconstruction takes the dense S2 (sigma = 1.8 omega, Ns = 8)."""
+    dwf, dims, ns, m0, mq = gpu_lib, (4, 4, 2, 4), 8, 1.8, 0.1
+    om, sg = np.ones(ns), 1.8 * np.ones(ns)
+    U = inputs.gauge_field(dims, 0.3, seed=64)
+    eta = inputs.gaussian_source(dims, ns, seed=65)
+    with dwf.Context(dims, ns, m0, mq, om, sg, U) as ctx:
+        psi, st = dwf.dwf_solve(ctx.h, eta, tol=1e-10)
+    res = np.linalg.norm(eta - oracle.dfull(dims, ns, U, m0, mq, om, sg, psi)) / np.linalg.norm(eta)
+    assert st["converged"] == 1 and res <= 1e-10
 
 
 def test_whole_operator_where_the_dense_corner_cancels(gpu_lib):
