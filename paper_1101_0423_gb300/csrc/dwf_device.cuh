@@ -33,7 +33,9 @@ template <int P> struct PT;
 // LREALS: reals per link; SITE_LREALS: reals per site's eight links, padding included
 template <> struct PT<P_F64> {
   using real = double; using chunk = double2; using lreal = double;
-  static constexpr int NCH = 12, RPC = 2, LREALS = 18, SITE_LREALS = 8 * 18; static constexpr bool HALF = false;
+  // a site's links padded by 16 bytes to 1168 (73 x 16), so that the sites of a warp read their
+  // broadcast entries from different banks
+  static constexpr int NCH = 12, RPC = 2, LREALS = 18, SITE_LREALS = 8 * 18 + 2; static constexpr bool HALF = false;
 };
 template <> struct PT<P_F32> {
   using real = float; using chunk = float4; using lreal = float;
@@ -366,9 +368,9 @@ __device__ __forceinline__ void hop_dir_raw(f2 (&acc)[12], const f2 (&ps)[12], c
 // neighbour is stored as a spinor or, in a halo slot, as its projection.
 
 constexpr int FX_EMIN = 80, FX_EMAX = 2000;
-// int4 per site of the fixed-point links: 8 links x 9 entries {re hi, re lo, im hi, im lo}, and
-// one of padding, so that the sites of a warp read from different banks
-constexpr int FX_SITE_I4 = 73;
+// int4 per site of the fixed-point links: 8 links x 9 entries {re hi, re lo, im hi, im lo}, in the
+// place of the links as copied
+constexpr int FX_SITE_I4 = PT<P_F64>::SITE_LREALS / 2;
 
 // V = x 2^(1075 + L - E), truncated, as V = hi 2^30 + lo; E is at least x's exponent field (an x
 // above it gives 0, and so do FP64 zeros and denormals)
@@ -481,18 +483,19 @@ __device__ __forceinline__ double from_fixed(long long a, int k) {
   return u ? __longlong_as_double((long long)r) : 0.0;
 }
 
-// a link row (three complex entries) in units of 2^-60, split as above; false if its 2-norm is
-// out of bounds or not a number
-__device__ __forceinline__ bool link_row_fixed(const double *w, int4 *o) {
+// a link row (three complex entries) to units of 2^-60, split as above, in place: an entry {re hi,
+// re lo, im hi, im lo} takes its two doubles' 16 bytes; false if its 2-norm is out of bounds or
+// not a number
+__device__ __forceinline__ bool link_row_fixed(double2 *w) {
   float n2 = 0.f;
 #pragma unroll
   for (int b = 0; b < 3; ++b) {
-    const double re = w[2 * b], im = w[2 * b + 1];
-    n2 += (float)re * (float)re + (float)im * (float)im;
-    int4 v;
-    to_fixed<8>(re, 1023, v.x, v.y);
-    to_fixed<8>(im, 1023, v.z, v.w);
-    o[b] = v;
+    const double2 u = w[b];
+    n2 += (float)u.x * (float)u.x + (float)u.y * (float)u.y;
+    int xh, xl, yh, yl;
+    to_fixed<8>(u.x, 1023, xh, xl);
+    to_fixed<8>(u.y, 1023, yh, yl);
+    w[b] = make_double2(__hiloint2double(xl, xh), __hiloint2double(yl, yh));
   }
   return n2 <= 1.01f;
 }

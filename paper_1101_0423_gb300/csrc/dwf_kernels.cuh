@@ -248,7 +248,7 @@ __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~size_t(
 // (links and indices arrive by TMA bulk copies).  FP32 kernels use the links as copied (padded
 // to 80 bytes, so the nine complex entries are five aligned float4); the 16-bit forms rebuild
 // each link's third row and expand the tile's links into that same FP32 form; FP64 kernels
-// convert them to fixed point once for the Ns threads of a site.  The M5 staging rows overlay
+// convert them to fixed point in place, once for the Ns threads of a site.  The M5 staging rows overlay
 // everything from offset 64 on (kernels with an M5 epilogue have one buffer, which is dead by
 // then; a CTA that walks several tiles refills it after the barrier and the proxy fence at the
 // top of the tile loop).  Shared memory is kept small on purpose: what the CTAs leave of the
@@ -270,10 +270,11 @@ template <int P> struct HopSmem {
   // stores fall in distinct bank groups; sites padded by another 16 bytes
   static constexpr int ROW = 24 + 16 / (int)sizeof(RL);
   __host__ __device__ static size_t stage(int spb, int Ns) { return (size_t)spb * (Ns * ROW * sizeof(RL) + 16); }
-  // FP32 links are used as copied; the other forms are expanded
-  // (16-bit: to the FP32 form; FP64: to the fixed-point form)
-  static constexpr bool EXPAND = P != P_F32;
-  static constexpr int EXP_SITE_BYTES = 16 * (F2 ? LINK_SITE_F4 : FX_SITE_I4);
+  // FP32 links are used as copied, FP64 links converted in place (a copy of their own left one
+  // CTA per SM at Ns = 1, and C at 16^4 x 1 in FP64 took 330 us instead of 225); 16-bit ones are
+  // expanded to the FP32 form
+  static constexpr bool EXPAND = PT<P>::HALF;
+  static constexpr int EXP_SITE_BYTES = 16 * LINK_SITE_F4;
   __host__ __device__ static size_t off_k(int spb, int Ns, int nb, bool has_m) {
     const size_t e = off_exp(spb, nb) + (EXPAND ? (size_t)spb * EXP_SITE_BYTES : 0);
     const size_t st = has_m ? 64 + stage(spb, Ns) : 0;
@@ -352,7 +353,8 @@ __device__ __forceinline__ void s_recurrence(double2 *col, int step, const doubl
   }
 }
 
-// the hop sum of one (site, s) in plain FP64 (fields or links out of the fixed-point range)
+// the hop sum of one (site, s) in plain FP64 (fields or links out of the fixed-point range), with
+// the site's links as stored in global memory
 template <int P>
 __device__ __noinline__ void hop_site_f64(const Field in, const int *nb, int s, int Ns, const double *links, double *out) {
   double acc[24];
@@ -535,10 +537,10 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
     bool slow_tile = false;  // FP64: a link is out of the fixed-point range
     if constexpr (!F2) {
       bool bad = false;
-      int4 *sI = reinterpret_cast<int4 *>(sP);
+      double2 *sW = reinterpret_cast<double2 *>(sLb(bsel));
       for (int r = tid; r < nsite * 24; r += nthr) {
         const int l = r / 24, row = r - 24 * l;
-        bad |= !link_row_fixed(sL + (size_t)l * T::SITE_LREALS + row * 6, sI + (size_t)l * FX_SITE_I4 + row * 3);
+        bad |= !link_row_fixed(sW + (size_t)l * FX_SITE_I4 + row * 3);
       }
       slow_tile = __syncthreads_or(bad);
     } else if constexpr (SM::EXPAND) {
@@ -594,7 +596,7 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
         for (int c = 0; c < 24; ++c) ai[c] = 0;
         int ex = FX_EMIN;
         bool ok = !slow_tile;
-        const int4 *myW = reinterpret_cast<const int4 *>(sP) + (size_t)sl * FX_SITE_I4;
+        const int4 *myW = reinterpret_cast<const int4 *>(sL) + (size_t)sl * FX_SITE_I4;
 #pragma unroll
         for (int mu = 0; mu < 4; ++mu) {
 #pragma unroll
@@ -615,7 +617,7 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
           for (int c = 0; c < 24; ++c) acc[c] = from_fixed(ai[c], ex - 57);  // times 2^(ex - 1080)
         } else {
           R slow[24];
-          hop_site_f64<P>(F(a.in), nb, s, Ns, sL + (size_t)sl * T::SITE_LREALS, slow);
+          hop_site_f64<P>(F(a.in), nb, s, Ns, static_cast<const R *>(a.gauge) + (size_t)cb * T::SITE_LREALS, slow);
 #pragma unroll
           for (int c = 0; c < 24; ++c) acc[c] = slow[c];
         }

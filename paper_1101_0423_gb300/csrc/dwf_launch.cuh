@@ -22,12 +22,12 @@ inline int sites_per_block(int Ns) {
 }
 
 // sites per CTA of k_hop, whose CTA is (Ns, spb): 128 threads measured best at Ns = 16
-// (against 256 and 512 threads, and 64 and 96, for the FP32 hop kernels)
+// (against 256 and 512 threads, and 64 and 96, for the FP32 hop kernels); in FP64 at most 62
+// sites, of whose links (1168 bytes each) three CTAs fit on an SM
 inline int hop_sites_per_block(int P, int Ns) {
-  const int target = 128;
-  (void)P;
+  const int target = 128, most = P == P_F64 ? 62 : 64;
   int spb = target / Ns;
-  if (spb > 64) spb = 64;
+  if (spb > most) spb = most;
   return spb < 1 ? 1 : spb;
 }
 
