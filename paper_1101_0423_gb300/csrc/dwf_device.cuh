@@ -369,7 +369,7 @@ __device__ __forceinline__ void hop_dir_raw(f2 (&acc)[12], const f2 (&ps)[12], c
 
 constexpr int FX_EMIN = 80, FX_EMAX = 2000;
 // int4 per site of the fixed-point links: 8 links x 9 entries {re hi, re lo, im hi, im lo}, in the
-// place of the links as copied
+// place of the links as copied; the site's padding, 0 as stored, is set where a row is out of bounds
 constexpr int FX_SITE_I4 = PT<P_F64>::SITE_LREALS / 2;
 
 // V = x 2^(1075 + L - E), truncated, as V = hi 2^30 + lo; E is at least x's exponent field (an x

@@ -534,15 +534,14 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
         if (it > 0) prefetch_ops(tile);
       }
     }
-    bool slow_tile = false;  // FP64: a link is out of the fixed-point range
     if constexpr (!F2) {
-      bool bad = false;
       double2 *sW = reinterpret_cast<double2 *>(sLb(bsel));
       for (int r = tid; r < nsite * 24; r += nthr) {
         const int l = r / 24, row = r - 24 * l;
-        bad |= !link_row_fixed(sW + (size_t)l * FX_SITE_I4 + row * 3);
+        double2 *const site = sW + (size_t)l * FX_SITE_I4;
+        if (!link_row_fixed(site + row * 3)) reinterpret_cast<int4 *>(site)[FX_SITE_I4 - 1].x = 1;
       }
-      slow_tile = __syncthreads_or(bad);
+      __syncthreads();
     } else if constexpr (SM::EXPAND) {
       // 16-bit links: rebuild row 3 and expand each link into the padded FP32 form
       for (int l = tid; l < nsite * 8; l += nthr) {
@@ -591,12 +590,12 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
 #pragma unroll
         for (int q = 0; q < 12; ++q) upk2(ac2[q], acc[2 * q], acc[2 * q + 1]);
       } else {
+        const int4 *myW = reinterpret_cast<const int4 *>(sL) + (size_t)sl * FX_SITE_I4;
         long long ai[24];
 #pragma unroll
         for (int c = 0; c < 24; ++c) ai[c] = 0;
         int ex = FX_EMIN;
-        bool ok = !slow_tile;
-        const int4 *myW = reinterpret_cast<const int4 *>(sL) + (size_t)sl * FX_SITE_I4;
+        bool ok = true;
 #pragma unroll
         for (int mu = 0; mu < 4; ++mu) {
 #pragma unroll
@@ -612,6 +611,9 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
             }
           }
         }
+        // a site with a link row out of bounds takes plain FP64, its neighbours in the tile do not:
+        // a site's result does not depend on the tile it is in
+        ok &= myW[FX_SITE_I4 - 1].x == 0;
         if (ok) {
 #pragma unroll
           for (int c = 0; c < 24; ++c) acc[c] = from_fixed(ai[c], ex - 57);  // times 2^(ex - 1080)

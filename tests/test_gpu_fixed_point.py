@@ -180,3 +180,21 @@ def test_whole_operator_where_the_dense_corner_cancels(gpu_lib):
         got = dwf.dwf_apply_eo(ctx.h, dwf.OP_DFULL, dwf.PREC_F64, 1, x)
     want = oracle.dfull(dims, ns, U, m0, mq, om, sg, x)
     assert np.abs(got - want).max() <= 100 * 1.2e-16 * 500 * np.abs(x).max()
+
+
+def test_link_out_of_bounds_changes_its_own_sites_only(gpu_lib):
+    """Which arithmetic a site takes depends on its own links: one link scaled out of the checked
+    bound leaves every output but those at its two ends bit for bit as it was, whatever tile
+    they share with them."""
+    U = inputs.gauge_field(DIMS, 0.5, seed=66).reshape(-1, 4, 18)
+    x = inputs.gaussian_source(DIMS, NS, seed=67)
+    before = run(gpu_lib, U.reshape(-1), x)
+    nx, ny, nz, nt = DIMS
+    for site, mu in ((0, 0), (nx * ny * nz + 5, 3), (37, 1)):
+        V = U.copy()
+        V[site, mu] *= 40.0
+        at = [site % nx, site // nx % ny, site // (nx * ny) % nz, site // (nx * ny * nz)]
+        at[mu] = (at[mu] + 1) % DIMS[mu]
+        ends = {site, at[0] + nx * (at[1] + ny * (at[2] + nz * at[3]))}
+        differ = set(np.flatnonzero((run(gpu_lib, V.reshape(-1), x) != before).any((1, 2))))
+        assert differ == {e for e in ends if inputs.site_parity(DIMS)[e] == 0}
