@@ -360,14 +360,31 @@ __device__ __forceinline__ void hop_dir_raw(f2 (&acc)[12], const f2 (&ps)[12], c
 // three 64-bit multiply-adds per real product; the dropped Wl Vl are below one unit each.
 // Bounds: a link row's 2-norm is at most sqrt(1.01) (checked; SU(3) rows have norm 1), so a
 // row's result is below sqrt(1.01 * 6) 2^58 < 2^59.4 and the sum over eight directions below
-// 2^62.4; the cross terms are below 6 (2^60 + 2^58) < 2^63.  An error of about one unit per
-// direction is 2^-56 of the largest |h|: below FP64's own rounding of the same sums
-// (2^-53 of each partial sum).  Links or neighbours outside the bounds (not finite, or
-// exponents outside [FX_EMIN, FX_EMAX]) take the FP64 arithmetic (hop_site_f64).
-// Neighbour sums therefore do not depend on the order of the sites of a tile or on whether a
-// neighbour is stored as a spinor or, in a halo slot, as its projection.
+// 2^62.4; the cross terms are below 6 (2^60 + 2^58) < 2^63.  The error is about one unit per
+// direction, 2^-56 of the largest |h| of the (site, s): half of FP64's own rounding of the
+// same sums by norm, on Gaussian fields; single components that are far smaller are looked
+// after below (FX_SEEN).  Links or neighbours outside the bounds (not finite, or exponents
+// outside [FX_EMIN, FX_EMAX]) take the FP64 arithmetic (hop_site_f64).  Which arithmetic a (site,
+// s) takes, and its result, follow from its own links and neighbours alone: not from the order
+// of the sites or the tile it is in, nor from whether a neighbour is stored as a spinor or, in
+// a halo slot, as its projection.
 
 constexpr int FX_EMIN = 80, FX_EMAX = 2000;
+
+// The unit follows the largest |h| among all twelve reals and eight neighbours, so a colour and
+// spin far below that one would keep few digits where the links do not mix it with the large ones
+// (unit or diagonal links).  A complex component of the result is therefore `seen` (a bit of
+// FX_SEEN each, colour + 3 spin) once a backward hop adds at least 2^53 units to it, against an
+// error of one unit a hop (root mean square; ten at most): no more than FP64 makes of the same
+// terms.  (E grows by two bits at least; the first such growth keeps what was seen, a second or
+// a larger one does not.)  Components that are not seen then count as such if they are 2^53 in
+// the result, or if fixed_loses finds that their terms' sizes are or that they have no term;
+// else the (site, s) takes plain FP64.  Testing the four backward hops finds all components of
+// Gaussian fields on SU(3) links but for one (site, s) in 40,000 (D^EO on 16^4 x 16
+// 352 -> 361 us; a field that falls by e a slice 351 -> 513).  2^54 would send one warp in eight of a
+// Gaussian field to fixed_loses (436 us), without a smaller root-mean-square error.
+constexpr unsigned FX_SEEN = 0xfff, FX_GREW = 0x1000, FX_BAD = 0x2000;
+constexpr int FX_SEEN_HI = 1 << 21;  // 2^53 in the upper word
 // int4 per site of the fixed-point links: 8 links x 9 entries {re hi, re lo, im hi, im lo}, in the
 // place of the links as copied; the site's padding, 0 as stored, is set where a row is out of bounds
 constexpr int FX_SITE_I4 = PT<P_F64>::SITE_LREALS / 2;
@@ -388,6 +405,11 @@ __device__ __forceinline__ void to_fixed(double x, int E, int &hi, int &lo) {
 // c + a b, the full 64-bit product
 __device__ __forceinline__ long long mad_w(int a, int b, long long c) { return (long long)a * b + c; }
 
+// either real is 2^53 units or more
+__device__ __forceinline__ bool fx_big(long long re, long long im) {
+  return (((unsigned)(int)(re >> 32) + FX_SEEN_HI) | ((unsigned)(int)(im >> 32) + FX_SEEN_HI)) >= 2u * FX_SEEN_HI;
+}
+
 // h_j = psi_up + S A psi_dn of direction MU (spin projection), FP64; one multiply-add a real (the
 // FP64 pipe issues DFMA faster than DADD, and a product with +-1 is exact)
 template <int MU>
@@ -405,29 +427,31 @@ __device__ __forceinline__ void project_f64(const double (&ps)[24], double S, do
     }
 }
 
-// acc += (1 + S g_MU) W psi in units of 2^(E - 1080); W: the link's nine entries; returns
-// false if a value is outside the fixed-point range (acc is then meaningless)
+// acc += (1 + S g_MU) W psi in units of 2^(E - 1080); W: the link's nine entries; st: FX_SEEN,
+// FX_GREW, FX_BAD (a value is outside the fixed-point range, acc is then meaningless)
 template <int MU>
-__device__ __forceinline__ bool hop_dir_fixed(long long (&acc)[24], int &E, const double (&ps)[24], const int4 *W,
-                                              const bool back) {
+__device__ __forceinline__ void hop_dir_fixed(long long (&acc)[24], int &E, unsigned &st, const double (&ps)[24],
+                                              const int4 *W, const bool back) {
   double h[12];
   project_f64<MU>(ps, back ? 1.0 : -1.0, h);
   int em = 0;
 #pragma unroll
   for (int q = 0; q < 12; ++q) em = max(em, __double2hiint(h[q]) & 0x7fffffff);
   em >>= 20;
-  bool ok = em <= FX_EMAX;
+  if (em > FX_EMAX) st |= FX_BAD;
   if (__builtin_expect(em < FX_EMIN, 0)) {  // all zero (nothing to add), or too small for the fixed-point range
     unsigned any = 0;
 #pragma unroll
     for (int q = 0; q < 12; ++q) any |= (unsigned)(__double2hiint(h[q]) << 1) | (unsigned)__double2loint(h[q]);
-    ok = any == 0;
+    if (any) st |= FX_BAD;
   }
   if (__builtin_expect(em > E, 0)) {
     const int d = min(em + 1 - E, 63);
 #pragma unroll
     for (int c = 0; c < 24; ++c) acc[c] >>= d;
     E = em + 1;
+    if (d == 2 && !(st & FX_GREW)) st |= FX_GREW;
+    else st &= FX_BAD;
   }
   int ph[6], pl[6], qh[6], ql[6], nh[6], nl[6];  // real parts, imaginary parts, - imaginary parts
 #pragma unroll
@@ -458,6 +482,7 @@ __device__ __forceinline__ bool hop_dir_fixed(long long (&acc)[24], int &E, cons
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
         if (ad_col(MU, k) != j) continue;
+        if (back && fx_big(re, im)) st |= 1u << (a + 3 * j) | 1u << (a + 3 * (2 + k));
         const int dn = 2 * (a + 3 * (2 + k)), p = ad_ph(MU, k);
         // S phase (re + i im): phase 0: 1, 1: i, 2: -1, 3: -i
         const long long vr = (p & 1) ? im : re, vi = (p & 1) ? re : im;
@@ -466,7 +491,6 @@ __device__ __forceinline__ bool hop_dir_fixed(long long (&acc)[24], int &E, cons
       }
     }
   }
-  return ok;
 }
 
 // a 2^(k - 1023), rounded to nearest even: as (double)a times a power of two, without the two

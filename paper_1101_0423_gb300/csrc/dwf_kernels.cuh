@@ -353,10 +353,75 @@ __device__ __forceinline__ void s_recurrence(double2 *col, int step, const doubl
   }
 }
 
-// the hop sum of one (site, s) in plain FP64 (fields or links out of the fixed-point range), with
-// the site's links as stored in global memory
+// whether the fixed-point sum of one (site, s) with exponent E loses a component that is not in
+// `seen`: it has a term, and the sizes of its terms, |link entry| |h| with the larger of either's real
+// and imaginary part, add up to less than 2^53 units (links: as stored in global memory; the
+// sizes in FP32, no instruction for the FP64 pipe but the projections)
 template <int P>
-__device__ __noinline__ void hop_site_f64(const Field in, const int *nb, int s, int Ns, const double *links, double *out) {
+__device__ __forceinline__ bool fixed_loses(const Field in, const int *nb, int s, int Ns, const double *links, int E,
+                                            unsigned seen) {
+  // the larger of |x| and |y| times 2^(shift + 896), rounded down to 20 bits (0 below FP32's
+  // range), and whether either is nonzero
+  auto size = [](double x, double y, int shift, bool &any) {
+    const int xh = __double2hiint(x) & 0x7fffffff, yh = __double2hiint(y) & 0x7fffffff, m = max(xh, yh);
+    any = (xh | yh | __double2loint(x) | __double2loint(y)) != 0;
+    const int e = (m >> 20) + shift;
+    return e > 0 ? __int_as_float(e << 23 | (m & 0xfffff) << 3) : 0.f;
+  };
+  float sum[12];
+#pragma unroll
+  for (int q = 0; q < 12; ++q) sum[q] = 0.f;
+  unsigned has = 0;
+#pragma unroll 1
+  for (int d = 0; d < 8; ++d) {
+    const int mu = d & 3;
+    const double S = d < 4 ? -1.0 : 1.0;
+    double ps[24], h[12], W[18];
+    load_sp<P>(in, nb[d], s, Ns, ps);
+    load_link<P>(links + d * PT<P>::LREALS, W);
+    switch (mu) {
+      case 0: project_f64<0>(ps, S, h); break;
+      case 1: project_f64<1>(ps, S, h); break;
+      case 2: project_f64<2>(ps, S, h); break;
+      default: project_f64<3>(ps, S, h); break;
+    }
+    float hs[6], ws[9];  // h in 2^53 units (times 2^(1080 - 53 - E)), W
+    bool hn[6], wn[9];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) hs[q] = size(h[2 * q], h[2 * q + 1], 1080 - 53 - 896 - E, hn[q]);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) ws[q] = size(W[2 * q], W[2 * q + 1], -896, wn[q]);
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        float t = 0.f;
+        bool any = false;
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+          t += ws[3 * a + b] * hs[b + 3 * j];
+          any |= wn[3 * a + b] && hn[b + 3 * j];
+        }
+        const bool k0 = ad_col(mu, 0) == j;  // the lower spin that this upper one's term also goes to
+        sum[a + 3 * j] += t;
+        sum[a + 6] += k0 ? t : 0.f;
+        sum[a + 9] += k0 ? 0.f : t;
+        if (any) has |= 1u << (a + 3 * j) | 1u << (a + (k0 ? 6 : 9));
+      }
+  }
+#pragma unroll
+  for (int q = 0; q < 12; ++q)
+    if (sum[q] >= 1.f) seen |= 1u << q;
+  return (has & ~seen) != 0;
+}
+
+// the hop sum of one (site, s) in plain FP64 (fields or links out of the fixed-point range), with
+// the site's links as stored in global memory; out holds the fixed-point sum, which stays where
+// it loses nothing
+template <int P>
+__device__ __noinline__ void hop_site_f64(const Field in, const int *nb, int s, int Ns, const double *links, int E,
+                                          unsigned fx, double *out) {
+  if (!(fx & FX_BAD) && ((fx & FX_SEEN) == FX_SEEN || !fixed_loses<P>(in, nb, s, Ns, links, E, fx))) return;
   double acc[24];
 #pragma unroll
   for (int c = 0; c < 24; ++c) acc[c] = 0;
@@ -595,7 +660,7 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
 #pragma unroll
         for (int c = 0; c < 24; ++c) ai[c] = 0;
         int ex = FX_EMIN;
-        bool ok = true;
+        unsigned fx = 0;
 #pragma unroll
         for (int mu = 0; mu < 4; ++mu) {
 #pragma unroll
@@ -604,22 +669,28 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
             load_sp<P>(F(a.in), nb[mu + 4 * back], s, Ns, ps);
             const int4 *W = myW + 9 * (mu + 4 * back);
             switch (mu) {
-              case 0: ok &= hop_dir_fixed<0>(ai, ex, ps, W, back); break;
-              case 1: ok &= hop_dir_fixed<1>(ai, ex, ps, W, back); break;
-              case 2: ok &= hop_dir_fixed<2>(ai, ex, ps, W, back); break;
-              default: ok &= hop_dir_fixed<3>(ai, ex, ps, W, back); break;
+              case 0: hop_dir_fixed<0>(ai, ex, fx, ps, W, back); break;
+              case 1: hop_dir_fixed<1>(ai, ex, fx, ps, W, back); break;
+              case 2: hop_dir_fixed<2>(ai, ex, fx, ps, W, back); break;
+              default: hop_dir_fixed<3>(ai, ex, fx, ps, W, back); break;
             }
           }
         }
         // a site with a link row out of bounds takes plain FP64, its neighbours in the tile do not:
         // a site's result does not depend on the tile it is in
-        ok &= myW[FX_SITE_I4 - 1].x == 0;
-        if (ok) {
+        if (myW[FX_SITE_I4 - 1].x) fx |= FX_BAD;
+        if ((fx & (FX_SEEN | FX_BAD)) == FX_SEEN || (ex == FX_EMIN && !(fx & FX_BAD))) {
 #pragma unroll
           for (int c = 0; c < 24; ++c) acc[c] = from_fixed(ai[c], ex - 57);  // times 2^(ex - 1080)
         } else {
           R slow[24];
-          hop_site_f64<P>(F(a.in), nb, s, Ns, static_cast<const R *>(a.gauge) + (size_t)cb * T::SITE_LREALS, slow);
+#pragma unroll
+          for (int q = 0; q < 12; ++q) {
+            slow[2 * q] = from_fixed(ai[2 * q], ex - 57);
+            slow[2 * q + 1] = from_fixed(ai[2 * q + 1], ex - 57);
+            if (fx_big(ai[2 * q], ai[2 * q + 1])) fx |= 1u << q;
+          }
+          hop_site_f64<P>(F(a.in), nb, s, Ns, static_cast<const R *>(a.gauge) + (size_t)cb * T::SITE_LREALS, ex, fx, slow);
 #pragma unroll
           for (int c = 0; c < 24; ++c) acc[c] = slow[c];
         }
