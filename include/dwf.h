@@ -261,23 +261,23 @@ dwf_status dwf_propagator_dev(dwf_ctx *ctx, const int x0[4], const dwf_solve_par
  * start-up -- and for paths that must not meet the device-wide synchronisation that a
  * cudaMalloc or cudaFree can bring).
  * Applies DWF_OP_DEO, DOE, M5, M5T, C, CDAG or CCDAG exactly as dwf_apply_eo_dev does, with
- * the same arguments, but takes every work field, the scalar block and the reduction
- * scratch from one static device array of 64 MiB compiled into the library (held on every
- * GPU that loads the library until the process exits) and calls no cudaMalloc, cudaFree or
+ * the same arguments, but takes every work field and the scalar block from one static
+ * device array of 64 MiB compiled into the library (held on every GPU that loads the
+ * library until the process exits) and calls no cudaMalloc, cudaFree or
  * other allocating routine.  The caller still passes the input and output arrays.  Limits
  * and behaviour:
- *   - five work fields plus the partial sums must fit in 64 MiB: about 5 * 24 * Ns * V4/2
+ *   - five work fields plus 8 bytes per CTA must fit in 64 MiB: about 5 * 24 * Ns * V4/2
  *     reals of the precision (FP32: Ns * V4/2 <= ~135,000; FP64: <= ~67,000, e.g. 8^4 x 16);
  *     larger lattices return DWF_EINVAL with the byte count in dwf_last_error;
  *   - the gauge field of `prec` must already exist (dwf_load_gauge builds FP64 and FP32; one
  *     dwf_apply_eo_dev call builds a 16-bit form), else DWF_EINVAL;
  *   - set-up: the first call on a context looks up the array's device address
  *     (cudaGetSymbolAddress) with the context's device current;
- *   - the call returns when its work is done: it synchronises `stream` and copies the
- *     kernels' 4-byte error word to the host (DWF_ETIMEOUT if a bounded device-side wait
+ *   - the call returns when its work is done: it synchronises `stream` and looks at the
+ *     kernels' error word in pinned host memory (DWF_ETIMEOUT if a bounded device-side wait
  *     gave up);
- *   - every call shares the one array, which keeps the last call's contents; the call clears
- *     what must start at zero itself.  Calls that overlap on the GPU (two streams, two
+ *   - every call shares the one array, which keeps the last call's contents (nothing in it
+ *     has to start at zero).  Calls that overlap on the GPU (two streams, two
  *     contexts, or two host threads) race on the array and must be serialised by the
  *     caller.  The context's own scratch is not used, so other calls on the context do not
  *     touch the array. */

@@ -2113,16 +2113,16 @@ extern "C" dwf_status dwf_propagator(dwf_ctx *c, const int x0[4], const dwf_solv
 // ====================================================================== allocation-free variant
 //
 // dwf_apply_eo_dev_static is dwf_apply_eo_dev for the Schur-parity operators with every
-// work field (packed input and output, three intermediates), the CG scalar block and the
-// reduction scratch (block partial sums and the last-block ticket) taken from one static
-// device array, so a call never allocates.  It is for callers that cannot let a library
+// work field (packed input and output, three intermediates) and the scalar block taken from
+// one static device array, so a call never allocates.  It is for callers that cannot let a library
 // allocate device memory: applications whose device memory is owned by their own pool
 // allocator (a framework's caching allocator that already holds the GPU's memory) or held
 // to a fixed budget decided at start-up, and paths that must not meet the device-wide
 // synchronisation a cudaMalloc or cudaFree can bring.  The array is a file-scope
 // __device__ variable, so every GPU that loads the library holds it until the process
-// exits.  The call touches no mutable state of the context (its device address of the
-// array aside), so other work on the same context is not redirected to the array.
+// exits.  Of the context's mutable state the call touches the array's device address
+// and an error word of its own, so other work on the same context is not redirected to the
+// array.
 
 namespace {
 
@@ -2153,7 +2153,8 @@ extern "C" dwf_status dwf_apply_eo_dev_static(dwf_ctx *c, int op, int prec, int 
                 "the gauge field of this precision is not built yet (dwf_load_gauge builds FP64 and FP32; "
                 "one dwf_apply_eo_dev call in a 16-bit precision builds that form)");
 
-  // carve five fields, the scalar block, the partial sums and the ticket out of the array
+  // carve five fields and the scalar block out of the array; the size limit is that of the
+  // interface, which also counts block partial sums (these operators take no reduction)
   const size_t n = (size_t)c->h * c->Ns;
   const size_t data_b = round256(n * site_bytes(prec));
   const size_t nrm_b = prec >= P_F16 ? round256(n * sizeof(float)) : 0;
@@ -2183,20 +2184,16 @@ extern "C" dwf_status dwf_apply_eo_dev_static(dwf_ctx *c, int op, int prec, int 
     cur += nrm_b;
   }
   CGScalars *sc = reinterpret_cast<CGScalars *>(cur);
-  cur += round256(sizeof(CGScalars));
-  double *part = reinterpret_cast<double *>(cur);
-  cur += round256(max_blocks * sizeof(double));
-  unsigned *ticket = reinterpret_cast<unsigned *>(cur);
 
   cudaStream_t st = stream ? (cudaStream_t)stream : c->stream;
-  // the array keeps the previous call's contents: nothing here reads the scalars, no launch
-  // takes a reduction (so the ticket is not used), and errors come through host memory
+  // the array keeps the previous call's contents: nothing here reads the scalars, and errors
+  // come through host memory
   c->h_err[1] = 0;
   const Geom g = geom(c);
   Field &in = f[0], &out = f[1], &tA = f[2], &tB = f[3], &tC = f[4];
   const int inpar = op == DWF_OP_DEO ? 1 : op == DWF_OP_DOE ? 0 : parity;
   const int outpar = op == DWF_OP_DEO ? 0 : op == DWF_OP_DOE ? 1 : parity;
-  // the hop launches of this call, with the reduction scratch of the array
+  // the hop launches of this call, with the scalar block of the array
   auto hop_s = [&](int outp, int epi, Field x, Field y, Field o, bool m5, bool trans, double coef) -> cudaError_t {
     HopArgs a = hop_args(c, prec, outp);
     a.in = x;
@@ -2205,8 +2202,8 @@ extern "C" dwf_status dwf_apply_eo_dev_static(dwf_ctx *c, int op, int prec, int 
     if (m5) set_m5(a, c, prec, trans);
     a.coef = coef;
     a.sc = sc;
-    a.partials = part;
-    a.ticket = ticket;
+    a.partials = nullptr;
+    a.ticket = nullptr;
     a.host_err = c->h_err + 1;
     a.fin = FIN_NONE;
     a.pdl = 1;
