@@ -641,11 +641,13 @@ dwf_status dwf_create(const int dims[4], int Ns, double m0, double mq, const dou
           kd[(size_t)chi * Ns * Ns + (size_t)t * Ns + s] = v;
           kf[(size_t)chi * Ns * Ns + (size_t)t * Ns + s] = (float)v;
         }
-    if ((e = dmalloc(&c->dmat[0][k], nm * sizeof(double), c->device, c->stream)) != cudaSuccess) return bail(e);
     if ((e = dmalloc(&c->dmat[1][k], nm * sizeof(float), c->device, c->stream)) != cudaSuccess) return bail(e);
-    if ((e = cudaMemcpyAsync(c->dmat[0][k], kd.data(), nm * sizeof(double), cudaMemcpyHostToDevice, c->stream)) !=
-        cudaSuccess)
-      return bail(e);
+    if (k < MK_W) {  // (FP64 takes the bidiagonal ones from their tables alone)
+      if ((e = dmalloc(&c->dmat[0][k], nm * sizeof(double), c->device, c->stream)) != cudaSuccess) return bail(e);
+      if ((e = cudaMemcpyAsync(c->dmat[0][k], kd.data(), nm * sizeof(double), cudaMemcpyHostToDevice, c->stream)) !=
+          cudaSuccess)
+        return bail(e);
+    }
     if ((e = cudaMemcpyAsync(c->dmat[1][k], kf.data(), nm * sizeof(float), cudaMemcpyHostToDevice, c->stream)) !=
         cudaSuccess)
       return bail(e);

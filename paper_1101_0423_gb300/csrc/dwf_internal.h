@@ -60,7 +60,8 @@ struct dwf_gauge {
 struct dwf_ctx : dwf::SMatrices {
   int dims[4];
   long V4, h;
-  // device matrices per arithmetic precision (0: double, 1: float), kernel order
+  // device matrices per arithmetic precision (0: double, none of the bidiagonal ones; 1: float),
+  // kernel order
   void *dmat[2][dwf::MK_COUNT] = {};
   double *drec[dwf::MK_COUNT] = {};  // recurrence tables (FP64); null where there is none
   int *d_nbr[2] = {nullptr, nullptr};
