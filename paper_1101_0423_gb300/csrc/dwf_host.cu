@@ -1083,9 +1083,12 @@ struct UseSlot {
 //   p = r + beta p, w = M5^T g5 p | t = -1/2 M5^T H w | q = p + 1/2 g5 H t, |q|^2
 //   u = -1/2 M5 H q | Ap = q + 1/2 M5 H u, r -= alpha Ap, x += alpha p, |r|^2, beta
 dwf_status cg_iteration(dwf_ctx *c, cudaStream_t st, const SolveState &S, const Slots &sl, int it) {
-  // Where the fields leave L2 behind (129 MB), successive kernels walk the sites in opposite
-  // directions, so that each begins with what its predecessor wrote and read last (16^3x32x16,
-  // 100 MB a field: 424 -> 415 us an iteration); smaller fields stay in L2 in any order
+  // Where a row's fields leave L2 behind (129 MB for the seven of an iteration), successive kernels
+  // walk the sites in opposite directions, so that each begins with what its predecessor wrote
+  // and read last.  An iteration in one and the other order: 36 MB a field (16^4 x 12) 209 and 199
+  // us, 48 MB 243 and 233, 72 MB 372 and 360, 100 MB 426 and 416; 24 MB 136 and 135, 3 MB 36.6 and
+  // 37.6.  The rows of a batch follow one another, and 12 of 2 to 15 MB a field take the same time
+  // either way (876 and 877 us at 15 MB), so only one row's field counts
   const int flip = field_bytes(c, S.prec) > ((size_t)32 << 20);
   int rev = flip & it;
   const int P = S.prec;
