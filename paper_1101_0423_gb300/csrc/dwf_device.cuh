@@ -381,7 +381,7 @@ constexpr int FX_EMIN = 80, FX_EMAX = 2000;
 // the result, or if fixed_loses finds that their terms' sizes are or that they have no term;
 // else the (site, s) takes plain FP64.  Testing the four backward hops finds all components of
 // Gaussian fields on SU(3) links but for one (site, s) in 40,000 (D^EO on 16^4 x 16
-// 352 -> 361 us; a field that falls by e a slice 351 -> 513).  2^54 would send one warp in eight of a
+// 352 -> 359 us; a field that falls by e a slice 353 -> 450).  2^54 would send one warp in eight of a
 // Gaussian field to fixed_loses (436 us), without a smaller root-mean-square error.
 constexpr unsigned FX_SEEN = 0xfff, FX_GREW = 0x1000, FX_BAD = 0x2000;
 constexpr int FX_SEEN_HI = 1 << 21;  // 2^53 in the upper word

@@ -421,7 +421,13 @@ __device__ __forceinline__ bool fixed_loses(const Field in, const int *nb, int s
 template <int P>
 __device__ __noinline__ void hop_site_f64(const Field in, const int *nb, int s, int Ns, const double *links, int E,
                                           unsigned fx, double *out) {
-  if (!(fx & FX_BAD) && ((fx & FX_SEEN) == FX_SEEN || !fixed_loses<P>(in, nb, s, Ns, links, E, fx))) return;
+  if (!(fx & FX_BAD)) {
+    // components of 2^53 units or more in the sum
+    for (int q = 0; q < 12; ++q)
+      if ((max(__double2hiint(out[2 * q]) & 0x7fffffff, __double2hiint(out[2 * q + 1]) & 0x7fffffff) >> 20) >= E - 4)
+        fx |= 1u << q;  // 2^(53 + E - 1080)
+    if ((fx & FX_SEEN) == FX_SEEN || !fixed_loses<P>(in, nb, s, Ns, links, E, fx)) return;
+  }
   double acc[24];
 #pragma unroll
   for (int c = 0; c < 24; ++c) acc[c] = 0;
@@ -679,17 +685,12 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
         // a site with a link row out of bounds takes plain FP64, its neighbours in the tile do not:
         // a site's result does not depend on the tile it is in
         if (myW[FX_SITE_I4 - 1].x) fx |= FX_BAD;
-        if ((fx & (FX_SEEN | FX_BAD)) == FX_SEEN || (ex == FX_EMIN && !(fx & FX_BAD))) {
 #pragma unroll
-          for (int c = 0; c < 24; ++c) acc[c] = from_fixed(ai[c], ex - 57);  // times 2^(ex - 1080)
-        } else {
+        for (int c = 0; c < 24; ++c) acc[c] = from_fixed(ai[c], ex - 57);  // times 2^(ex - 1080)
+        if (__builtin_expect((fx & (FX_SEEN | FX_BAD)) != FX_SEEN && (ex != FX_EMIN || (fx & FX_BAD)), 0)) {
           R slow[24];
 #pragma unroll
-          for (int q = 0; q < 12; ++q) {
-            slow[2 * q] = from_fixed(ai[2 * q], ex - 57);
-            slow[2 * q + 1] = from_fixed(ai[2 * q + 1], ex - 57);
-            if (fx_big(ai[2 * q], ai[2 * q + 1])) fx |= 1u << q;
-          }
+          for (int c = 0; c < 24; ++c) slow[c] = acc[c];
           hop_site_f64<P>(F(a.in), nb, s, Ns, static_cast<const R *>(a.gauge) + (size_t)cb * T::SITE_LREALS, ex, fx, slow);
 #pragma unroll
           for (int c = 0; c < 24; ++c) acc[c] = slow[c];
