@@ -602,7 +602,7 @@ def main():
                          "launch configuration (a short program for profiler captures): one solve first "
                          "picks the tuned launch shapes, then the applications run inside a profiler "
                          "range (capture with ncu --profile-from-start off)")
-    ap.add_argument("--apply-prec", choices=("f32", "f16", "bf16"), default="f32",
+    ap.add_argument("--apply-prec", choices=("f32", "f16", "bf16", "f64"), default="f32",
                     help="arithmetic form of --apply-ccdag")
     ap.add_argument("--configs", action="store_true",
                     help="only the per-configuration table: every workload at its real size, iterations, "
@@ -625,11 +625,13 @@ def main():
         y = torch.empty_like(x)
         with dwf.Context(DIMS, NS, M0, MQ, om, sg, inputs.gauge_field(DIMS, EPS, seed=SEED)) as ctx:
             stream = torch.cuda.current_stream()
-            prec = {"f32": dwf.PREC_F32, "f16": dwf.PREC_F16, "bf16": dwf.PREC_BF16}[args.apply_prec]
-            # the benchmark's solve tunes the launch shapes the applications then use
+            prec = {"f32": dwf.PREC_F32, "f16": dwf.PREC_F16, "bf16": dwf.PREC_BF16,
+                    "f64": dwf.PREC_F64}[args.apply_prec]
+            # the benchmark's solve tunes the launch shapes the applications then use (FP64 has
+            # one shape, its solve runs in FP32)
             eta = torch.from_numpy(inputs.gaussian_source(DIMS, NS, seed=SEED)).cuda()
-            dwf.dwf_solve_dev(ctx.h, eta, torch.empty_like(eta), stream=stream, inner_prec=prec,
-                              mode=dwf.MODE_RELIABLE)
+            dwf.dwf_solve_dev(ctx.h, eta, torch.empty_like(eta), stream=stream,
+                              inner_prec=dwf.PREC_F32 if prec == dwf.PREC_F64 else prec, mode=dwf.MODE_RELIABLE)
             stream.synchronize()
             torch.cuda.profiler.start()
             for _ in range(args.apply_ccdag):
