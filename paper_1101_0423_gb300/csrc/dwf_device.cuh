@@ -96,9 +96,10 @@ enum { RS_NONE = 0, RS_DELTA = 1, RS_TARGET = 2, RS_CAP = 3, RS_DIVERGED = 4, RS
 // their writes are visible.  The trigger stands at the end of a kernel's main work: there the
 // set-up hides behind the last CTAs and the reduction's tail (FP32 CG iteration at 8^4x16: 40.8
 // -> 36.2 us, at 16^3x32x16 429 -> 423 us).  At the start of the kernels it let later kernels'
-// CTAs pile up on whatever SM had room (51.7 and 468 us).  Nothing a predecessor writes is read, and nothing at all is written, before
-// pdl_wait(); field loads are plain (ld.global.nc promises data that is constant for the whole
-// launch, which such a launch cannot).  Without the launch attribute both are no-ops.
+// CTAs pile up on whatever SM had room (51.7 and 468 us).  Nothing a predecessor writes is
+// read, and nothing at all is written, before pdl_wait(); field loads are plain (ld.global.nc
+// promises data that is constant for the whole launch, which such a launch cannot).  Without
+// the launch attribute both are no-ops.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -451,13 +451,13 @@ __device__ __noinline__ void hop_site_f64(const Field in, const int *nb, int s, 
 // k_hop: one thread per (site, s), CTA = (Ns, spb) = one tile of spb sites at a time: one tile
 // per CTA, or a persistent grid of as many CTAs as fit on the GPU at once, walking all tiles
 // (the default of the FP32 and 16-bit kernels without an M5 epilogue; the autotuner may choose
-// either for every kernel of the inner CG).  Per tile: eight gathers of the neighbours' spinors (Eq. 12), the hop sum in packed FP32 pairs or
-// FP64 fixed point, the epilogue.  The FP64
+// either for every kernel of the inner CG).  Per tile: eight gathers of the neighbours' spinors
+// (Eq. 12), the hop sum in packed FP32 pairs or FP64 fixed point, the epilogue.  The FP64
 // forms (fixed-point products, FP64 projections and M5) are capped at 128 registers, four CTAs
 // per SM: a CTA's M5 phase keeps the FP64 pipe busy while others are in their integer hop
-// phase (C C^dag in FP64 at 16^3x32x16: 11.0 ms with the products in FP64, now 2.8 ms, 5 %
+// phase (C C^dag in FP64 at 16^3x32x16: 11.0 ms with the products in FP64, now 2.75 ms, 5 %
 // less than with three CTAs of 168 registers).  They wait as much on the FP64 pipe's latency
-// (57 % busy) as on issue (33 %): 16 warps per SM.
+// (58 % busy) as on issue (33 %): 16 warps per SM.
 template <int P, int EPI, int NSC>
 __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_hop(const HopArgs a) {
   // one right-hand side of a batch per grid row; fields are offset where they are used, so
@@ -1106,7 +1106,7 @@ __global__ void __launch_bounds__(256) k_smix(const SmixArgs a) {
 
 // FP64 matrices along s as recurrences (S_PLAIN, S_G5, S_CGP; RC_A): four FP64 operations a
 // real against Ns for the dense rows of k_smix, which the FP64 pipe bounded (16^3x32x16: M5^T
-// 693 us dense, 216 us so).  A CTA of (Ns, spb) threads puts its sites' columns (16 bytes x Ns, one
+// 693 us dense, 210 us so).  A CTA of (Ns, spb) threads puts its sites' columns (16 bytes x Ns, one
 // pair of reals) into shared memory in coalesced chunks, one thread runs each column, and the
 // result leaves in chunks again.  Columns are an odd number of 16-byte units apart, so that
 // the eight columns of a quarter-warp fall in distinct banks.
@@ -1178,7 +1178,8 @@ __global__ void __launch_bounds__(256) k_srec(const SmixArgs a) {
 
 // FP64 S_DUAL with two cyclic bidiagonal matrices (omega + sigma L and (d - m0)(omega + sigma L)
 // + 1 - L of Eq. 5, or 1 and d - m0): tables of RC_A with the diagonal in A and the factor of L
-// at the next step in D (W of the last step at the corner).  Two multiply-adds a real and matrix; each slice reads its neighbour along s through L1.
+// at the next step in D (W of the last step at the corner).  Two multiply-adds a real and
+// matrix; each slice reads its neighbour along s through L1.
 __global__ void __launch_bounds__(256) k_sdual(const SmixArgs a);
 
 // ------------------------------------------------------------------ per-(site, s) vector kernels

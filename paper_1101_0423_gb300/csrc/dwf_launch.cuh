@@ -177,7 +177,7 @@ template <int P>
 cudaError_t smix_launch(int mode, const SmixArgs &a, cudaStream_t st) {
   if constexpr (P == P_F64) {
     // as recurrences; dense only where a matrix has no table as accurate as its rows (16^3x32x16:
-    // 216 us against 693 us)
+    // 210 us against 693 us)
     switch (mode) {
       case S_PLAIN: return a.rec ? srec_go<S_PLAIN>(a, st) : smix_go<P, S_PLAIN>(a, st);
       case S_G5: return a.rec ? srec_go<S_G5>(a, st) : smix_go<P, S_G5>(a, st);
