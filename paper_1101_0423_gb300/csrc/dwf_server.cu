@@ -28,6 +28,7 @@
 #include <vector>
 
 #include "../../include/dwf.h"
+#include "dwf_device.cuh"
 
 namespace {
 
@@ -69,10 +70,11 @@ struct Entry {
 size_t site_bytes(int prec) { return prec == DWF_PREC_F64 ? 192 : prec == DWF_PREC_F32 ? 96 : 52; }
 
 // device memory of a gauge ensemble once resident: the FP64 copy and the doubled link
-// forms in FP64, FP32 and 16 bits
+// forms in FP64, FP32 and 16 bits, as the kernels store a site's links
 size_t gauge_bytes(const int dims[4]) {
+  using namespace dwf;
   const size_t V4 = (size_t)dims[0] * dims[1] * dims[2] * dims[3], h = V4 / 2;
-  return V4 * 72 * 8 + 2 * h * (1152 + 656 + 192);
+  return V4 * 72 * 8 + 2 * h * (PT<P_F64>::SITE_LREALS * 8 + PT<P_F32>::SITE_LREALS * 4 + PT<P_F16>::SITE_LREALS * 2);
 }
 
 // device memory a context needs for a batch of `rows` solves (tables, solver fields,

@@ -1,4 +1,4 @@
-"""Orderings in the kernels' source (csrc/dwf_kernels.cuh) that no run can be relied on to show."""
+"""Orderings and sizes in the source (csrc) that no run can be relied on to show."""
 import os
 import re
 
@@ -20,3 +20,12 @@ def test_refilled_link_buffer_is_fenced_against_its_staging_rows():
     # no other bulk copy reuses bytes that ordinary stores wrote: the first copy of a CTA and
     # the double-buffered ones, whose buffers are only read
     assert loop.count("issue(") == 2 and src.count("issue(") == 3
+
+
+def test_server_counts_the_links_as_the_kernels_store_them():
+    """The server's budget takes a gauge ensemble's bytes from the link layouts' own constants, so
+    that a padded site is counted with its padding."""
+    src = open(os.path.join(os.path.dirname(KERNELS), "dwf_server.cu")).read()
+    body = re.search(r"size_t gauge_bytes\(.*?\n}\n", src, re.S).group()
+    assert [p in body for p in ("PT<P_F64>::SITE_LREALS * 8", "PT<P_F32>::SITE_LREALS * 4", "PT<P_F16>::SITE_LREALS * 2")] == [True] * 3
+    assert not re.search(r"\b(1152|656|192)\b", body)
