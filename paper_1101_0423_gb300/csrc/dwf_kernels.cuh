@@ -665,7 +665,7 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
         long long ai[24];
 #pragma unroll
         for (int c = 0; c < 24; ++c) ai[c] = 0;
-        int ex = FX_EMIN;
+        int ex = FX_EMIN - 1;  // no neighbour but zeros so far
         unsigned fx = 0;
 #pragma unroll
         for (int mu = 0; mu < 4; ++mu) {
@@ -687,7 +687,7 @@ __global__ void __launch_bounds__(P == P_F64 ? 128 : 256, P == P_F64 ? 4 : 0) k_
         if (myW[FX_SITE_I4 - 1].x) fx |= FX_BAD;
 #pragma unroll
         for (int c = 0; c < 24; ++c) acc[c] = from_fixed(ai[c], ex - 57);  // times 2^(ex - 1080)
-        if (__builtin_expect((fx & (FX_SEEN | FX_BAD)) != FX_SEEN && (ex != FX_EMIN || (fx & FX_BAD)), 0)) {
+        if (__builtin_expect((fx & (FX_SEEN | FX_BAD)) != FX_SEEN && (ex >= FX_EMIN || (fx & FX_BAD)), 0)) {
           R slow[24];
 #pragma unroll
           for (int c = 0; c < 24; ++c) slow[c] = acc[c];

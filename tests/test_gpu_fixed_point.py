@@ -248,6 +248,19 @@ def test_components_of_different_size(gpu_lib, links, decades):
     assert np.sqrt((rel ** 2).mean()) <= 2.3e-16
 
 
+def test_components_at_the_smallest_exponent(gpu_lib):
+    """Upper spins whose largest component has the smallest exponent of the fixed-point range (2^-943),
+    on unit links: the components a billion times smaller keep FP64's accuracy too."""
+    U = np.ascontiguousarray(np.broadcast_to(np.eye(3, dtype=complex), (int(np.prod(DIMS)) * 4, 3, 3))).view(float).reshape(-1)
+    rng = np.random.RandomState(5)
+    x = rng.uniform(1.0, 1.999, (int(np.prod(DIMS)), NS, 12, 2)) * 2.0 ** -943
+    x[:, :, 1:6] *= 1e-9
+    x[:, :, 6:] = 0.0
+    got, want = run(gpu_lib, U, x.reshape(-1)), oracle.hop(DIMS, NS, U, 0, x.reshape(-1)).reshape(-1, NS, 24)
+    terms = np.repeat(hop_terms(U, x.reshape(-1)).reshape(-1, NS, 12), 2, axis=2)
+    assert (np.abs(got - want) <= 3.8e-14 * terms)[inputs.site_parity(DIMS) == 0].all()
+
+
 def test_components_without_terms_are_zero(gpu_lib):
     """A field with one spin and colour on links that do not mix colours: every component that no
     term reaches is exactly 0, the others are as in FP64."""
