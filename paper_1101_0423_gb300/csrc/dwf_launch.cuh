@@ -148,11 +148,21 @@ cudaError_t hop_launch(int epi, const HopArgs &a, cudaStream_t st) {
   return cudaErrorInvalidValue;
 }
 
+// sites per CTA of k_smix.  CTAs of about 128 threads for small and middle Ns: the p-update's three
+// operands in flight take 88 registers, five CTAs per SM (4^4x8: 31.2 -> 29.4 us an iteration, 12
+// rows of 8^4x8: 77.1 -> 75.2 ms a solve).  Every CTA stages the matrices, 2 Ns^2 reals (S_DUAL
+// 4), which at large Ns cost more than its sites: there 256 threads, so twice the sites.  128 and
+// 256 threads on 12^3x16 in FP32: D at Ns = 28 317 and 316 us, 32 331 and 326, 48 630 and 538, 64
+// 1005 and 808; M5 at 32 118 and 118.5, 33 140 and 137, 64 268 and 256; an iteration at 32 227 and
+// 230, 40 366 and 368, 48 459 and 460 (bf16 500 and 492), 64 650 and 631.
+inline int smix_sites_per_block(int P, int mode, int Ns) {
+  const int wide_from = mode == S_DUAL ? 32 : mode == S_CGP ? 48 : 33;
+  return P != P_F64 && Ns >= wide_from ? 256 / Ns : sites_per_block(Ns);
+}
+
 template <int P, int MODE>
 cudaError_t smix_go(const SmixArgs &a, cudaStream_t st) {
-  // 128 threads: the p-update's three operands in flight take 88 registers, five CTAs per SM
-  // (4^4x8: 31.2 -> 29.4 us an iteration, 12 rows of 8^4x8: 77.1 -> 75.2 ms a solve)
-  const int spb = sites_per_block(a.Ns);
+  const int spb = smix_sites_per_block(P, MODE, a.Ns);
   const size_t smem = smix_smem_bytes<P>(spb, a.Ns, MODE == S_DUAL);
   static SmemOptIn optin;
   const cudaError_t e = allow_smem(optin, k_smix<P, MODE>, smem);
