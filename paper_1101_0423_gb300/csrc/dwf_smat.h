@@ -248,8 +248,8 @@ inline bool recurrence_table(const SMatrices &c, int kind, int chi, double *T) {
 // latter's own few roundings and y_0's rounding, carried along s by the product of the E, stays
 // below the largest entry's.  Where sigma > omega that product grows along s and the dense rows
 // are the more accurate.  Tight tables err less than the rows (root mean square over random
-// fields, in units of 2^-52 of the result: Shamir 0.24 against 0.5-0.9 for Ns = 4 to 64, Borici
-// 0.27-0.29 against 0.4-0.9, cosine 0.29-0.36 against 0.9-1.2).
+// fields, in units of 2^-52 of the result, M5, M5^T and S1 at Ns = 4 to 64: Shamir 0.24 against
+// 0.5-0.9, Borici 0.27-0.29 against 0.4-1.0, cosine 0.30-0.37 against 0.6-1.1).
 inline bool build_recurrences(SMatrices *c) {
   const int Ns = c->Ns;
   std::vector<double> u(Ns), v(Ns);
